@@ -242,7 +242,7 @@ HP_API int hp_sweep(hp_handle* h, int32_t n_mcs, void* stream);
  * 26-neighbour lattice, lean 3D windows (64 x 44, 40, 36, 32: variants 8-11;
  * every random number drawn while the window is in flight).  Until a variant is
  * chosen, a handle sweeps with the fastest measured for its kind of lattice:
- * variant 11 in 3D with material points, 8 in 3D without, 4 in 2D.
+ * variant 11 in 3D, 4 in 2D.
  * hp_sweep_variants: how many exist for `nbr`.
  * hp_set_sweep_variant: choose one (HP_ERR_ARG if not built for the handle's
  * field mode).  hp_sweep_autotune: time every variant for n_mcs MCS on a

@@ -66,27 +66,47 @@ __device__ __forceinline__ uint4 philox10(uint32_t k0, uint32_t k1, uint4 c) {
     return c;
 }
 
-// The same rounds with the ten round keys given (rk[2r], rk[2r+1] for round r,
-// as philox_round_keys makes them), so that a kernel can take them from its
-// launch parameters instead of stepping the key in every thread.
-__device__ __forceinline__ uint4 philox10_keyed(const uint32_t* rk, uint4 c) {
-#pragma unroll
-    for (int r = 0; r < 10; ++r) {
-        const uint32_t lo0 = 0xD2511F53u * c.x, hi0 = __umulhi(0xD2511F53u, c.x);
-        const uint32_t lo1 = 0xCD9E8D57u * c.z, hi1 = __umulhi(0xCD9E8D57u, c.z);
-        c = make_uint4(hi1 ^ c.y ^ rk[2 * r], lo1, hi0 ^ c.w ^ rk[2 * r + 1], lo0);
-    }
-    return c;
-}
+// Words 0 and 1 of the draws of one MCS (counter unit, 0, sweep, colour; tag 0),
+// with everything that the whole launch shares taken out of the rounds.  Sites
+// have indices below 2^31, so counter word 1 is 0; then round 1's second product
+// and round 2's first depend on the seed and the sweep alone, and of round 10
+// only words 0 and 1 are wanted: 34 operations a draw where the ten full rounds
+// with stepped keys take about 60.
+struct SweepKey {
+    uint32_t z1;          // round 1: key of word 2 (the colour is added by xor)
+    uint32_t x2, z2, w2;  // round 2: what word 0 and word 2 are xored with, word 3
+    uint32_t rk[16];      // round keys of rounds 3 .. 10
+};
 
-__host__ __device__ inline void philox_round_keys(uint64_t seed, uint32_t rk[20]) {
+__host__ __device__ inline void sweep_key(uint64_t seed, uint32_t sweep, SweepKey* k) {
     uint32_t k0 = (uint32_t)seed, k1 = (uint32_t)(seed >> 32);
-    for (int r = 0; r < 10; ++r) {
-        rk[2 * r] = k0;
-        rk[2 * r + 1] = k1;
+    const uint64_t ps = (uint64_t)0xCD9E8D57u * sweep;
+    const uint32_t x1 = (uint32_t)(ps >> 32) ^ k0, y1 = (uint32_t)ps;
+    k->z1 = k1;
+    k0 += 0x9E3779B9u;
+    k1 += 0xBB67AE85u;
+    const uint64_t px = (uint64_t)0xD2511F53u * x1;
+    k->x2 = y1 ^ k0;
+    k->z2 = (uint32_t)(px >> 32) ^ k1;
+    k->w2 = (uint32_t)px;
+    for (int r = 0; r < 8; ++r) {
         k0 += 0x9E3779B9u;
         k1 += 0xBB67AE85u;
+        k->rk[2 * r] = k0;
+        k->rk[2 * r + 1] = k1;
     }
+}
+
+__device__ __forceinline__ uint2 sweep_draw(const SweepKey& k, uint32_t unit, uint32_t colour) {
+    const uint32_t z1 = __umulhi(0xD2511F53u, unit) ^ (k.z1 ^ colour), w1 = 0xD2511F53u * unit;
+    uint4 c = make_uint4(__umulhi(0xCD9E8D57u, z1) ^ k.x2, 0xCD9E8D57u * z1, w1 ^ k.z2, k.w2);
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+        const uint32_t lo0 = 0xD2511F53u * c.x, hi0 = __umulhi(0xD2511F53u, c.x);
+        const uint32_t lo1 = 0xCD9E8D57u * c.z, hi1 = __umulhi(0xCD9E8D57u, c.z);
+        c = make_uint4(hi1 ^ c.y ^ k.rk[2 * r], lo1, hi0 ^ c.w ^ k.rk[2 * r + 1], lo0);
+    }
+    return make_uint2(c.x, c.y);
 }
 
 __device__ __forceinline__ uint4 draw(uint64_t seed, uint64_t unit, uint32_t step, uint32_t tag, uint32_t sub) {

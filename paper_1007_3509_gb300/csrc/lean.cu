@@ -1,30 +1,39 @@
 // Lean 3D kernel of the fused checkerboard sweep (Eq. (7), Sec. 4) for the
 // 26-neighbour simple cubic lattice, built to spend few instructions per
-// site-update.
+// site-update and to keep a warp from waiting for others.
 //
 // Colours c = (x&1) + 2(y&1) + 4(z&1): one MCS is two launches, the even planes
 // (colours 0-3, their z-neighbours the odd planes as they were) and then the odd
 // planes (colours 4-7, their z-neighbours the even planes as just updated).  One
-// CTA = one 64 x WY window of one plane with its two z-neighbour windows: q (and,
-// with material points, mp) of the three planes, filled by 16-byte asynchronous
-// copies that every thread issues (a few hundred small bulk copies from one warp
-// queue up behind each other in the copy engine; spread over all threads they
-// overlap the draws).  The window keeps a halo of four columns and two
-// rows on each side (the exact region of the four in-plane phases, as in the 2D
-// Moore tiles), so the core is (64 - 8) x (WY - 4).
+// CTA = one 64 x WY window of one plane: q of the plane and of its two
+// z-neighbours and, with material points, mp of the plane.  The window keeps a
+// halo of four columns and two rows on each side (the exact region of the four
+// in-plane phases, as in the 2D Moore tiles), so the core is (64 - 8) x (WY - 4).
 //
-// Three ideas keep the instruction count down:
-//  * every random number of the launch is drawn while the window is in flight:
-//    each thread owns a fixed set of sites of each phase (lane = column of the
-//    colour sub-grid, warp = rows) and keeps their neighbour choice k and
-//    acceptance draw u1 in registers, so Philox overlaps the memory latency;
-//  * there is no interior test: a site proposes its k-th neighbour's grain and
+// What the kernel is bound by: instructions and the latency of the few dependent
+// loads of a test, not memory.  What keeps both down:
+//  * every random number of the launch is drawn while the window is in flight and
+//    stays in registers (lane = column of the colour sub-grid);
+//  * there is no interior test: a site proposes its k-th neighbour's grain, and
 //    only proposals of another grain (about a fifth of the sites in a
-//    polycrystal) go on to a block-wide queue;
-//  * the queue is worked by consecutive threads (whole warps busy), which count
-//    both grains among the 26 neighbours with two shared loads per row and run
-//    the integer Metropolis test of Sec. 4.
-// Each phase is then: propose + enqueue, barrier, test + flip, barrier.
+//    polycrystal) are tested;
+//  * a warp owns whole rows.  Phases 0 and 1 (even rows) see the odd rows only as
+//    they arrived, and phases 2 and 3 the even rows only as phases 0 and 1 left
+//    them, so a warp queues and tests its own proposals phase after phase with no
+//    more than warp-level synchronisation; the block meets once, between phases 1
+//    and 2.  A block-wide queue (two block barriers per phase, half of the warps
+//    idle in every test) spent 3.7 of 10 stall cycles per instruction there;
+//  * four warps of WY / 8 row pairs each: about 28 of the 128 sites a warp looks
+//    at per phase go on to its test, one per lane, so a pass runs nearly full.
+//    With eight warps (14 proposals, two lanes to each) the same window took 66 %
+//    more instructions and 138 us where this takes 100;
+//  * the neighbour planes' material points are gathered for the proposals that
+//    point there instead of being staged: 37 KB of shared memory a block, six
+//    blocks on an SM (staged, 53 KB and four).
+// Measured on 512^3 (two launches per MCS), site-updates/s: point field 7.9e10 ->
+// 9.2e10, grain field 1.10e11 -> 1.25e11; 512 x 512 x 64, one launch, ncu: 113.6
+// -> 100.7 us and 10.0 -> 7.7 warp instructions per site-update with the point
+// field, 87.2 -> 77.8 us with the grain field.
 #include <string.h>
 
 #include <cudaTypedefs.h>
@@ -42,7 +51,8 @@ __device__ int g_lean_err;
 // the point that started at site p).
 struct alignas(64) LeanMaps {
     CUtensorMap q_in, q_nb, mp_in, mp_nb, tab;
-    int ok;   // 1: the q (and mp) descriptors are valid
+    int ok;   // 1: the q (and mp_in) descriptors are valid
+    int pfm;  // 1: `mp_nb` is valid (the neighbour planes' material points are prefetched into L2)
     int pf;   // 1: `tab` is valid (the field table is prefetched into L2)
 };
 
@@ -60,19 +70,25 @@ __device__ __forceinline__ void tma_prefetch_l2(const CUtensorMap* map, int x, i
 }
 
 
-template <int WY, bool HASMP>
+template <int WY, int FIELD, bool HASMP>
 struct LeanCfg {
-    static constexpr int kLT = 256, NW = kLT / 32;
+    static constexpr int NW = 4, kLT = 32 * NW;
     static constexpr int WX = 64, HX = 4, HY = 2, TX = WX - 2 * HX, TY = WY - 2 * HY;
-    static constexpr int PS = WX * WY;             // one plane window, ints
-    static constexpr int NA = HASMP ? 6 : 3;       // q(z-1) q(z) q(z+1) [mp(z-1) mp(z) mp(z+1)]
-    static constexpr int SX = WX / 2, SY = WY / 2, NSUB = SX * SY;  // sites of one colour in the window
-    static constexpr int PER = (NSUB + kLT - 1) / kLT;               // of them per thread
-    static_assert(SX == 32 && WY % 2 == 0 && TY % 2 == 0 && PER <= 4, "lean window shape");
-    // blocks per SM: shared memory allows 4 with the material-point planes when
-    // WY <= 32 (3 above), 5 without them
-    static constexpr int MINB = HASMP ? (WY <= 32 ? 4 : 3) : 5;
-    static constexpr size_t smem() { return 128 + 4 * (size_t)NA * PS + 8 * (size_t)NSUB + 4 * 32 + 4 * 4 + 8; }
+    static constexpr int PS = WX * WY;             // one plane window, sites
+    static constexpr int NA = HASMP ? 4 : 3;       // window arrays: q(z-1) q(z) q(z+1) [mp(z)]
+    static constexpr int SX = WX / 2, SY = WY / 2;                   // one colour's sites in the window
+    static constexpr int PER = (SY + NW - 1) / NW;                   // row pairs per warp
+    static constexpr int CAP = 32 * PER;                             // sites of one colour per warp
+    static_assert(SX == 32 && WY % 2 == 0 && TY % 2 == 0, "lean window shape");
+    // 64 x 32 is the fastest on every lattice measured (512^3, point field: 5.83
+    // ms for 4 MCS against 6.8, 7.0 and 7.5 ms of 36, 40 and 44 rows, whose row
+    // pairs do not share out evenly among four warps)
+    // shared memory: the window arrays | a proposal queue per warp | neighbour
+    // offsets | mbarrier
+    static constexpr size_t smem() { return 128 + 4 * (size_t)NA * PS + 8 * (size_t)(NW * CAP) + 4 * 28 + 8; }
+    // blocks per SM that the shared memory allows (228 KB, 1 KB of it per block taken)
+    static constexpr int FIT = (int)(228 * 1024 / (smem() + 1024));
+    static constexpr int MINB = FIT > 7 ? 7 : FIT;
     __host__ __device__ static constexpr int ylo(int p) { return 1 + (p >> 1); }
 };
 
@@ -97,56 +113,133 @@ __global__ void k_wait_probe(long long limit, int late) {
     wait_or_drain(mb, &g_lean_err, limit);
 }
 
+// a wrapped into [0, L), however far off (windows wider than the lattice)
+__device__ __noinline__ int wrap_any(int a, int L) { return wrapi(a, L); }
+
 // One window (tile `tile` of plane 2 zidx + a.zpar) of one lattice; maps NULL
 // when no window of this launch is copied by TMA boxes.
-// KEYED: the Philox round keys come from a.rk (launch parameters); otherwise
-// every thread steps the key from a.seed.
-template <int WY, int FIELD, bool HASMP, bool KEYED>
+template <int WY, int FIELD, bool HASMP>
+struct Lean {
+    using Cfg = LeanCfg<WY, FIELD, HASMP>;
+    static constexpr int WX = Cfg::WX, PS = Cfg::PS;
+    const PlaneArgs& a;
+    int32_t* Q;         // q of plane z (z-1 at -PS, z+1 at +PS)
+    int32_t* MP;        // mp of plane z
+    int x0, y0;
+    uint32_t lobase, hibase;  // first site of planes z-1, z+1
+    uint32_t tab_last;        // last index of the field table
+    bool fast;    // the window fits the lattice
+    bool inside;  // and does not cross its edge in x or y
+
+    __device__ __forceinline__ Lean(const PlaneArgs& a_) : a(a_) {}
+    __device__ __forceinline__ int gx_of(int col) const {
+        int v = x0 - 4 + col;
+        if (!inside) v = fast ? wrap1(v, a.Lx) : wrap_any(v, a.Lx);
+        return v;
+    }
+    __device__ __forceinline__ int gy_of(int r) const {
+        int v = y0 - 2 + r;
+        if (!inside) v = fast ? wrap1(v, a.Ly) : wrap_any(v, a.Ly);
+        return v;
+    }
+    // field table entry, the index clamped into the table
+    __device__ __forceinline__ int32_t field(int32_t i) const { return __ldg(a.table + min((uint32_t)i, tab_last)); }
+    // material point of the neighbour at offset o: of planes z-1 and z+1, which
+    // this launch does not change, from global memory
+    __device__ __forceinline__ int32_t mp_of(int pos, int o) const {
+        if (o >= -(PS / 2) && o <= PS / 2) return MP[pos + o];
+        const int n = pos + o + (o < 0 ? PS : -PS);
+        return __ldg(a.mp_nb + (o < 0 ? lobase : hibase) + (uint32_t)gx_of(n & (WX - 1)) +
+                     (uint32_t)a.Lx * (uint32_t)gy_of(n / WX));
+    }
+    // The Metropolis test of the proposal at pos (offset o, acceptance draw u1).
+    __device__ __forceinline__ void test(int pos, int o, uint32_t u1) const {
+        const int32_t* c = Q + pos;
+        const int32_t qi = c[0], qj = c[o];
+        int32_t mj = 0, bi = 0, bj = 0;
+        if (HASMP) mj = mp_of(pos, o);
+        if (FIELD) {
+            bi = field(FIELD == 2 ? MP[pos] : qi);
+            bj = field(FIELD == 2 ? mj : qj);
+        }
+        // all 27 sites of the neighbourhood: of each row the aligned pair with the
+        // site's column and the column on its other side; the site itself counts
+        // once among those of its own grain
+        const int32_t* pr = Q + (pos & ~1);
+        const int32_t* sg = c + ((pos & 1) ? 1 : -1);
+        int ni[3] = {0, -1, 0}, nj[3] = {0, 0, 0};  // per plane: six short chains of adds
+#pragma unroll
+        for (int dy = -1; dy <= 1; ++dy)
+#pragma unroll
+            for (int dz = 0; dz < 3; ++dz) {
+                const int2 v = *reinterpret_cast<const int2*>(pr + (dz - 1) * PS + dy * WX);
+                const int32_t w = sg[(dz - 1) * PS + dy * WX];
+                if (v.x == qi) ++ni[dz];
+                if (v.x == qj) ++nj[dz];
+                if (v.y == qi) ++ni[dz];
+                if (v.y == qj) ++nj[dz];
+                if (w == qi) ++ni[dz];
+                if (w == qj) ++nj[dz];
+            }
+        const int dn = (ni[0] + ni[1] + ni[2]) - (nj[0] + nj[1] + nj[2]);
+        if (metropolis(a.J * dn + (bj - bi), a.D, a.thr, u1)) {
+            Q[pos] = qj;
+            if (HASMP) MP[pos] = mj;
+        }
+    }
+};
+
+template <int WY, int FIELD, bool HASMP>
 __device__ __forceinline__ void lean_body(const PlaneArgs& a, const LeanMaps* maps, const int tile, const int zidx,
                                           unsigned char* raw) {
-    using Cfg = LeanCfg<WY, HASMP>;
-    constexpr int WX = Cfg::WX, PS = Cfg::PS, NA = Cfg::NA, NSUB = Cfg::NSUB, PER = Cfg::PER, kLT = Cfg::kLT;
-    constexpr int NW = Cfg::NW;
+    using L = Lean<WY, FIELD, HASMP>;
+    using Cfg = typename L::Cfg;
+    constexpr int WX = Cfg::WX, PS = Cfg::PS, NA = Cfg::NA, PER = Cfg::PER, CAP = Cfg::CAP;
+    constexpr int NW = Cfg::NW, kLT = Cfg::kLT;
+    constexpr bool EVEN = Cfg::SY % NW == 0;  // every warp has PER row pairs
     int32_t* base = reinterpret_cast<int32_t*>(raw + ((128u - (s_addr(raw) & 127u)) & 127u));
-    int32_t* Q = base + PS;                                       // q of plane z (z-1 at -PS, z+1 at +PS)
-    int32_t* MP = base + 4 * PS;                                  // mp of plane z, same layout
-    uint2* queue = reinterpret_cast<uint2*>(base + NA * PS);      // NSUB entries
-    int* off = reinterpret_cast<int*>(queue + NSUB);              // 26 neighbour offsets (+ pad)
-    int* qn = off + 32;                                           // 4 phase counters
-    unsigned long long* mbar = reinterpret_cast<unsigned long long*>(qn + 4);
-
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    L w(a);
+    w.Q = base + PS;
+    w.MP = base + 3 * PS;
+    uint2* queue = reinterpret_cast<uint2*>(base + NA * PS) + CAP * warp;  // this warp's: pos | offset << 16, u1
+    int* off = reinterpret_cast<int*>(base + NA * PS + 2 * CAP * NW);      // offset of neighbour k at [k + 1], 0 at [0]
+    unsigned long long* mbar = reinterpret_cast<unsigned long long*>(off + 28);
+
     const int ty = tile / a.tiles_x, tx = tile - ty * a.tiles_x;
-    const int x0 = tx * Cfg::TX, y0 = ty * Cfg::TY;
+    w.x0 = tx * Cfg::TX;
+    w.y0 = ty * Cfg::TY;
+    const int x0 = w.x0, y0 = w.y0;
     const int z = 2 * zidx + a.zpar;
-    const int zlo = wrapi(z - 1, a.Lz), zhi = wrapi(z + 1, a.Lz);
-    const int64_t sxy = (int64_t)a.Lx * a.Ly;
-    const bool fast = a.fast != 0;
-    auto gx_of = [&](int col) { return fast ? wrap1(x0 - 4 + col, a.Lx) : wrapi(x0 - 4 + col, a.Lx); };
-    auto gy_of = [&](int r) { return fast ? wrap1(y0 - 2 + r, a.Ly) : wrapi(y0 - 2 + r, a.Ly); };
-    auto src = [&](int arr) -> const int32_t* {
-        const int pl = arr % 3;
-        const int zz = pl == 0 ? zlo : (pl == 1 ? z : zhi);
-        if (arr < 3) return (pl == 1 ? a.q_in : a.q_nb) + sxy * zz;
-        return (pl == 1 ? a.mp_in : a.mp_nb) + sxy * zz;
-    };
+    const int zlo = z > 0 ? z - 1 : a.Lz - 1, zhi = z < a.Lz - 1 ? z + 1 : 0;
+    const uint32_t sxy = (uint32_t)a.Lx * (uint32_t)a.Ly;
+    const uint32_t zbase = sxy * (uint32_t)z;
+    w.lobase = sxy * (uint32_t)zlo;
+    w.hibase = sxy * (uint32_t)zhi;
+    w.tab_last = a.table_n - 1u;
+    w.fast = a.fast != 0;
+    w.inside = x0 >= 4 && x0 - 4 + WX <= a.Lx && y0 >= 2 && y0 - 2 + WY <= a.Ly;
 
     // ---- window in flight ----------------------------------------------------
     // A window inside the lattice arrives as one tiled TMA box per array (64 x WY
     // of plane z, one request each, completing on an mbarrier that warp 0 polls).
-    // A window that crosses the periodic edge is filled with 16-byte asynchronous
-    // copies issued by every thread (4 ints of one window row each: x0 - 4 and Lx
-    // are multiples of 4, so a chunk never straddles the edge).  Either way the
-    // copies land while the draws below run.
-    const bool vec = a.Lx % 4 == 0 && ((uintptr_t)a.q_in & 15u) == 0 && ((uintptr_t)a.q_nb & 15u) == 0 &&
-                     (!HASMP || (((uintptr_t)a.mp_in & 15u) == 0 && ((uintptr_t)a.mp_nb & 15u) == 0));
-    const bool boxed = vec && maps && maps->ok && x0 >= 4 && x0 - 4 + WX <= a.Lx && y0 >= 2 && y0 - 2 + WY <= a.Ly;
-    if (tid < 26) {
-        const int kk = tid + (tid >= 13);
-        off[tid] = (kk / 9 - 1) * PS + ((kk / 3) % 3 - 1) * WX + (kk % 3 - 1);
+    // A window that crosses the periodic edge is filled with asynchronous copies
+    // issued by every thread, 16 bytes where rows keep 16-byte boundaries (Lx % 4
+    // == 0) and 8 bytes otherwise (edges are even: x0 - 4 and Lx are multiples of
+    // the chunk, so no chunk straddles the edge; 250 x 198 x 130 with material
+    // points, 10 MCS: 3.28 ms with 4-byte loads and a modulo per coordinate, 1.20
+    // ms with this kernel).  Either way the copies land while the draws below run.
+    const uintptr_t low = (uintptr_t)a.q_in | (uintptr_t)a.q_nb | (HASMP ? (uintptr_t)a.mp_in : 0);
+    const bool v16 = a.Lx % 4 == 0 && (low & 15u) == 0, v8 = !v16 && (low & 7u) == 0;
+    const bool boxed = v16 && maps && maps->ok && w.inside;
+    if (tid < 27) {
+        const int k = tid - 1, kk = k + (k >= 13);
+        off[tid] = tid ? (kk / 9 - 1) * PS + ((kk / 3) % 3 - 1) * WX + (kk % 3 - 1) : 0;
     }
-    if (tid < 4) qn[tid] = 0;
     const uint32_t mb = s_addr(mbar);
+    auto src = [&](int arr) -> const int32_t* {
+        return arr == 0 ? a.q_nb + w.lobase : arr == 1 ? a.q_in + zbase : arr == 2 ? a.q_nb + w.hibase : a.mp_in + zbase;
+    };
     if (boxed) {
         if (tid == 0) {
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(mb) : "memory");
@@ -157,200 +250,167 @@ __device__ __forceinline__ void lean_body(const PlaneArgs& a, const LeanMaps* ma
             tma_box(s_addr(base), &maps->q_nb, xs, ys, zlo, mb);
             tma_box(s_addr(base + PS), &maps->q_in, xs, ys, z, mb);
             tma_box(s_addr(base + 2 * PS), &maps->q_nb, xs, ys, zhi, mb);
-            if (HASMP) {
-                tma_box(s_addr(base + 3 * PS), &maps->mp_nb, xs, ys, zlo, mb);
-                tma_box(s_addr(base + 4 * PS), &maps->mp_in, xs, ys, z, mb);
-                tma_box(s_addr(base + 5 * PS), &maps->mp_nb, xs, ys, zhi, mb);
+            if (HASMP) tma_box(s_addr(base + 3 * PS), &maps->mp_in, xs, ys, z, mb);
+            // The proposals look up the material points of the neighbour planes
+            // and the field of the window's material points.  A point moves only a
+            // few sites under grain growth, so most of them lie in the table's
+            // boxes at the window's own coordinates: start these towards L2 now.
+            if (HASMP && maps->pfm) {
+                tma_prefetch_l2(&maps->mp_nb, xs, ys, zlo);
+                tma_prefetch_l2(&maps->mp_nb, xs, ys, zhi);
             }
-            // The test stages look up the field of the window's material points.
-            // A point moves only a few sites under grain growth, so most of them
-            // lie in the table's boxes at the window's own coordinates: start
-            // those towards L2 now, a few thousand cycles before the lookups.
             if (FIELD == 2 && maps->pf) {
                 tma_prefetch_l2(&maps->tab, xs, ys, zlo);
                 tma_prefetch_l2(&maps->tab, xs, ys, z);
                 tma_prefetch_l2(&maps->tab, xs, ys, zhi);
             }
         }
-    } else if (vec) {
-        constexpr int CH = WX / 4;  // chunks per window row
-        for (int i = tid; i < NA * WY * CH; i += kLT) {
-            const int arr = i / (WY * CH), rem = i - arr * (WY * CH), r = rem / CH, c = rem - r * CH;
-            const int gx = fast ? wrap1(x0 - 4 + 4 * c, a.Lx) : wrapi(x0 - 4 + 4 * c, a.Lx);
-            const int32_t* g = src(arr) + (int64_t)a.Lx * gy_of(r) + gx;
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(s_addr(base + arr * PS + r * WX + 4 * c)),
-                         "l"(g) : "memory");
+    } else if (v16) {
+        const int c = 4 * (tid & 15), gx = w.gx_of(c);
+#pragma unroll
+        for (int r = tid >> 4; r < WY; r += kLT / 16) {
+            const uint32_t g = (uint32_t)gx + (uint32_t)a.Lx * (uint32_t)w.gy_of(r);
+#pragma unroll
+            for (int arr = 0; arr < NA; ++arr)
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(s_addr(base + arr * PS + r * WX + c)),
+                             "l"(src(arr) + g) : "memory");
         }
-        asm volatile("cp.async.commit_group;" ::: "memory");
+    } else if (v8) {
+        const int c = 2 * lane, gx = w.gx_of(c);
+        for (int r = warp; r < WY; r += NW) {
+            const uint32_t g = (uint32_t)gx + (uint32_t)a.Lx * (uint32_t)w.gy_of(r);
+#pragma unroll
+            for (int arr = 0; arr < NA; ++arr)
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(s_addr(base + arr * PS + r * WX + c)),
+                             "l"(src(arr) + g) : "memory");
+        }
+    } else {
+        for (int i = tid; i < PS; i += kLT) {
+            const uint32_t g = (uint32_t)w.gx_of(i & (WX - 1)) + (uint32_t)a.Lx * (uint32_t)w.gy_of(i / WX);
+#pragma unroll
+            for (int arr = 0; arr < NA; ++arr) base[arr * PS + i] = src(arr)[g];
+        }
     }
     // every thread sees the barrier initialised (and the offsets) before it waits
     __syncthreads();
 
     // ---- every draw of the launch, while the copies land -------------------
-    // site m of phase p for this thread: colour sub-grid column = lane, row
-    // j = warp + NW m; window column 2 lane + (p & 1), row 2 j + (p >> 1).  Its
-    // Philox unit gx + Lx (gy + Ly z) is a row base plus a column, each wrapped
-    // once per thread.  Whether the row lies in the phase's region is the same
-    // for the whole warp (a branch); whether the column does is a select, so a
-    // warp never diverges here (the few edge lanes draw and drop the result).
+    // Warp v owns the row pairs (2j, 2j + 1), j = v + NW m; lane = column of the
+    // colour sub-grid, so that the lane's sites of the pair are the four window
+    // positions (2 lane, 2 lane + 1) x (2j, 2j + 1), one of each phase.  A site's
+    // Philox unit is a row base plus a column, each wrapped once per thread.
+    // Whether the row lies in the phase's region is the same for the whole warp
+    // (a branch); whether the column does is a select.  A slot without a site
+    // gets choice 0 (offset 0): it proposes itself, which is no proposal.
     const uint32_t cz = 4u * (uint32_t)a.zpar;
-    const uint64_t gxc[2] = {(uint64_t)gx_of(2 * lane), (uint64_t)gx_of(2 * lane + 1)};
-    uint64_t rowb[PER][2];
+    const uint32_t gxc[2] = {(uint32_t)w.gx_of(2 * lane), (uint32_t)w.gx_of(2 * lane + 1)};
+    const int pos0 = 2 * warp * WX + 2 * lane;
+    uint32_t u1[4][PER];
+    uint32_t kk[2][PER];  // choices + 1 of phases 2r, 2r + 1 in bytes 0 and 1
 #pragma unroll
     for (int m = 0; m < PER; ++m) {
-        const int j = warp + NW * m;
 #pragma unroll
-        for (int r = 0; r < 2; ++r)
-            rowb[m][r] = j < Cfg::SY ? (uint64_t)a.Lx * ((uint64_t)gy_of(2 * j + r) + (uint64_t)a.Ly * (uint64_t)z) : 0;
-    }
-    uint32_t u1[4][PER];
-    uint32_t kk[4];
+        for (int r = 0; r < 2; ++r) {
+            const int y = 2 * (warp + NW * m) + r;
+            kk[r][m] = 0;
+            u1[2 * r][m] = u1[2 * r + 1][m] = 0;
+            if (y >= Cfg::ylo(2 * r) && y < WY - Cfg::ylo(2 * r)) {
+                const uint32_t rowb = zbase + (uint32_t)a.Lx * (uint32_t)w.gy_of(y);
 #pragma unroll
-    for (int p = 0; p < 4; ++p) {
-        kk[p] = 0;
-        const int x = 2 * lane + (p & 1), loy = Cfg::ylo(p);
-        const bool colok = x >= p + 1 && x < WX - p - 1;
-#pragma unroll
-        for (int m = 0; m < PER; ++m) {
-            const int j = warp + NW * m, y = 2 * j + (p >> 1);
-            u1[p][m] = 0;
-            if (j < Cfg::SY && y >= loy && y < WY - loy) {
-                const uint64_t unit = rowb[m][p >> 1] + gxc[p & 1];
-                const uint4 u =
-                    KEYED ? philox10_keyed(a.rk, make_uint4((uint32_t)unit, (uint32_t)(unit >> 32), a.sweep,
-                                                            (kTagSweep << 24) | (cz + (uint32_t)p)))
-                          : draw(a.seed, unit, a.sweep, kTagSweep, cz + (uint32_t)p);
-                u1[p][m] = u.y;
-                kk[p] |= (colok ? __umulhi(u.x, 26u) + 1u : 0u) << (8 * m);  // 0 marks "no site"
+                for (int px = 0; px < 2; ++px) {
+                    const int p = 2 * r + px, x = 2 * lane + px;
+                    const uint2 u = sweep_draw(a.key, rowb + gxc[px], cz + (uint32_t)p);
+                    u1[p][m] = u.y;
+                    kk[r][m] |= (x >= p + 1 && x < WX - p - 1 ? __umulhi(u.x, 26u) + 1u : 0u) << (8 * px);
+                }
             }
         }
     }
 
     if (boxed) {
         if (!wait_or_drain(mb, &g_lean_err)) return;
-    } else if (vec) {
+    } else {
         asm volatile("cp.async.wait_all;" ::: "memory");
         __syncthreads();
-    } else {
-        for (int i = tid; i < NA * PS; i += kLT) {
-            const int arr = i / PS, rem = i - arr * PS, r = rem / WX, c = rem - r * WX;
-            base[arr * PS + rem] = src(arr)[(int64_t)a.Lx * wrapi(y0 - 2 + r, a.Ly) + wrapi(x0 - 4 + c, a.Lx)];
-        }
-        __syncthreads();
     }
 
+    // ---- phases.  Sites of phases 0 and 1 share the even rows and meet phase 2's
+    // and 3's, in the odd rows, only as unchanged neighbours (and the other way
+    // round), so a warp runs phases 0 and 1 of its own rows on its own, and after
+    // one block barrier phases 2 and 3.
     const unsigned lt = (1u << lane) - 1u;
-    // kernel parameters of the test stage, once
-    const int32_t* __restrict__ ftab = a.table;
-    const uint32_t ftab_n = a.table_n;
-    const uint32_t* __restrict__ thr = a.thr;
-    const int32_t Jc = a.J, Dmax = a.D;
-    constexpr int SAFE = (WY / 2) * WX + WX / 2;  // a window position whose 26 neighbours all lie in the window
-#pragma unroll
+#pragma unroll 1
     for (int p = 0; p < 4; ++p) {
-        // ---- propose: the k-th neighbour's grain; queue those of another grain.
-        // An empty slot (kc = 0) reads at SAFE instead, so every lane loads and
-        // no branch is taken.
-        uint32_t e[PER];
-        unsigned bal[PER];
-        int tot = 0;
+        const int at = pos0 + (p >> 1) * WX + (p & 1), sh = 8 * (p & 1);
+        int n = 0;
 #pragma unroll
         for (int m = 0; m < PER; ++m) {
-            const uint32_t kc = (kk[p] >> (8 * m)) & 255u;
-            const int pos = (2 * (warp + NW * m) + (p >> 1)) * WX + 2 * lane + (p & 1);
-            const int k = kc ? (int)kc - 1 : 0;
-            const int pq = kc ? pos : SAFE;
-            const int32_t qa = Q[pq + off[k]], qb = Q[pq];
-            const bool pr = (kc != 0u) & (qa != qb);
-            e[m] = (uint32_t)pos | ((uint32_t)k << 16);
-            bal[m] = __ballot_sync(0xFFFFFFFFu, pr);
-            tot += __popc(bal[m]);
+            if (!EVEN && warp + NW * m >= Cfg::SY) continue;
+            const uint32_t kc = ((p & 2 ? kk[1][m] : kk[0][m]) >> sh) & 255u;
+            const uint32_t u = p & 2 ? (p & 1 ? u1[3][m] : u1[2][m]) : (p & 1 ? u1[1][m] : u1[0][m]);
+            const int pos = at + 2 * NW * m * WX, o = off[kc];
+            const bool pr = w.Q[pos + o] != w.Q[pos];
+            const unsigned bal = __ballot_sync(0xFFFFFFFFu, pr);
+            if (pr) queue[n + __popc(bal & lt)] = make_uint2((uint32_t)pos | ((uint32_t)o << 16), u);
+            n += __popc(bal);
         }
-        if (tot) {
-            int b0 = 0;
-            if (lane == 0) b0 = atomicAdd(qn + p, tot);
-            b0 = __shfl_sync(0xFFFFFFFFu, b0, 0);
-#pragma unroll
-            for (int m = 0; m < PER; ++m) {
-                if (bal[m] & (1u << lane)) queue[b0 + __popc(bal[m] & lt)] = make_uint2(e[m], u1[p][m]);
-                b0 += __popc(bal[m]);
-            }
+        __syncwarp();
+        for (int i = lane; i < n; i += 32) {
+            const uint2 e = queue[i];
+            w.test((int)(e.x & 0xFFFFu), (int)e.x >> 16, e.y);
         }
-        __syncthreads();
-        // ---- test: count both grains among the 26 neighbours, Metropolis ------
-        const int n = qn[p];
-        for (int i = tid; i < n; i += kLT) {
-            const uint2 w = queue[i];
-            const int pos = (int)(w.x & 0xFFFFu), o = off[w.x >> 16];
-            const int32_t* c = Q + pos;
-            const int32_t qi = c[0], qj = c[o];
-            int32_t mpj = 0, bi = 0, bj = 0;
-            if (HASMP) mpj = MP[pos + o];
-            if (FIELD == 1) { bi = tab(ftab, ftab_n, qi); bj = tab(ftab, ftab_n, qj); }
-            if (FIELD == 2) { bi = tab(ftab, ftab_n, MP[pos]); bj = tab(ftab, ftab_n, mpj); }
-            int so = 0, sn = 0;
-#pragma unroll
-            for (int dz = -1; dz <= 1; ++dz)
-#pragma unroll
-                for (int dy = -1; dy <= 1; ++dy) {
-                    const int32_t* r = c + dz * PS + dy * WX;
-                    int32_t v0, v1, v2;
-                    if (p & 1) {  // column odd: (x-1, x) is an aligned pair
-                        const int2 l = *reinterpret_cast<const int2*>(r - 1);
-                        v0 = l.x; v1 = l.y; v2 = r[1];
-                    } else {      // column even: (x, x+1) is an aligned pair
-                        const int2 h = *reinterpret_cast<const int2*>(r);
-                        v0 = r[-1]; v1 = h.x; v2 = h.y;
-                    }
-                    so += (v0 == qi) + (v2 == qi);
-                    sn += (v0 == qj) + (v2 == qj);
-                    if (dz != 0 || dy != 0) { so += v1 == qi; sn += v1 == qj; }
-                }
-            const int32_t d = Jc * (so - sn) + (bj - bi);
-            if (metropolis(d, Dmax, thr, w.y)) {
-                Q[pos] = qj;
-                if (HASMP) MP[pos] = mpj;
-            }
-        }
-        __syncthreads();
+        if (p == 1) __syncthreads(); else __syncwarp();
     }
 
-    // ---- write the core: rows [2, WY - 2), columns [4, WX - 4) ---------------
-    int32_t* qo = a.q_out + sxy * z;
-    int32_t* mpo = HASMP ? a.mp_out + sxy * z : nullptr;
-    constexpr int CQ = WX / 4 - 2;
-    for (int i = tid; i < Cfg::TY * CQ; i += kLT) {
-        const int cy = i / CQ, qq = 1 + (i - cy * CQ);
-        const int gx = x0 + 4 * (qq - 1), gy = y0 + cy;
-        if (gx >= a.Lx || gy >= a.Ly) continue;
-        const int li = (cy + 2) * WX + 4 * qq;
-        const int64_t o = gx + (int64_t)a.Lx * gy;
-        if (a.vec) {
-            *reinterpret_cast<int4*>(qo + o) = *reinterpret_cast<const int4*>(Q + li);
-            if (HASMP) *reinterpret_cast<int4*>(mpo + o) = *reinterpret_cast<const int4*>(MP + li);
-        } else {
+    // ---- write the warp's rows of the core: rows [2, WY - 2), columns [4, WX - 4)
+    int32_t* qo = a.q_out + zbase;
+    int32_t* mpo = HASMP ? a.mp_out + zbase : nullptr;
+    const uintptr_t lowo = (uintptr_t)a.q_out | (HASMP ? (uintptr_t)a.mp_out : 0);
+    const int wv = a.Lx % 4 == 0 && (lowo & 15u) == 0 ? 4 : (lowo & 7u) == 0 ? 2 : 1;
 #pragma unroll
-            for (int jx = 0; jx < 4; ++jx) {
-                if (gx + jx >= a.Lx) break;
-                qo[o + jx] = Q[li + jx];
-                if (HASMP) mpo[o + jx] = MP[li + jx];
+    for (int m = 0; m < PER; ++m) {
+        const int y = 2 * (warp + NW * m);  // 16-byte chunks: a half-warp per row; else a row after the other
+        if (wv == 4) {
+            const int yy = y + (lane >> 4), c = 4 * (lane & 15), gx = x0 + c - 4, gy = y0 + yy - 2;
+            if (yy < 2 || yy >= WY - 2 || c < 4 || c >= WX - 4 || gx >= a.Lx || gy >= a.Ly) continue;
+            const uint32_t o = (uint32_t)gx + (uint32_t)a.Lx * (uint32_t)gy;
+            *reinterpret_cast<int4*>(qo + o) = *reinterpret_cast<const int4*>(w.Q + yy * WX + c);
+            if (HASMP) *reinterpret_cast<int4*>(mpo + o) = *reinterpret_cast<const int4*>(w.MP + yy * WX + c);
+        } else {
+            const int c = 2 * lane, gx = x0 + c - 4;
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+                const int yy = y + r, gy = y0 + yy - 2, li = yy * WX + c;
+                if (yy < 2 || yy >= WY - 2 || c < 4 || c >= WX - 4 || gx >= a.Lx || gy >= a.Ly) continue;
+                const uint32_t o = (uint32_t)gx + (uint32_t)a.Lx * (uint32_t)gy;
+                if (wv == 2) {
+                    *reinterpret_cast<int2*>(qo + o) = *reinterpret_cast<const int2*>(w.Q + li);
+                    if (HASMP) *reinterpret_cast<int2*>(mpo + o) = *reinterpret_cast<const int2*>(w.MP + li);
+                } else {
+                    qo[o] = w.Q[li];
+                    qo[o + 1] = w.Q[li + 1];
+                    if (HASMP) {
+                        mpo[o] = w.MP[li];
+                        mpo[o + 1] = w.MP[li + 1];
+                    }
+                }
             }
         }
     }
 }
 
 template <int WY, int FIELD, bool HASMP>
-__global__ void __launch_bounds__(LeanCfg<WY, HASMP>::kLT, LeanCfg<WY, HASMP>::MINB)
+__global__ void __launch_bounds__(LeanCfg<WY, FIELD, HASMP>::kLT, LeanCfg<WY, FIELD, HASMP>::MINB)
     k_lean26(const __grid_constant__ PlaneArgs a, const __grid_constant__ LeanMaps maps) {
     extern __shared__ __align__(16) unsigned char raw[];
-    lean_body<WY, FIELD, HASMP, true>(a, &maps, (int)blockIdx.x, (int)blockIdx.y, raw);
+    lean_body<WY, FIELD, HASMP>(a, &maps, (int)blockIdx.x, (int)blockIdx.y, raw);
 }
 
 // Many independent lattices in one launch: block b belongs to the replica r
 // with start[r] <= b < start[r+1]; within it b - start[r] = zidx * tiles + tile.
 // Windows are filled by the asynchronous 16-byte copies.
 template <int WY, int FIELD, bool HASMP>
-__global__ void __launch_bounds__(LeanCfg<WY, HASMP>::kLT, HASMP ? 3 : 4)
+__global__ void __launch_bounds__(LeanCfg<WY, FIELD, HASMP>::kLT, LeanCfg<WY, FIELD, HASMP>::MINB)
     k_lean26_batch(const PlaneArgs* __restrict__ args, const int64_t* __restrict__ start, int R, uint32_t sweep_add) {
     extern __shared__ __align__(16) unsigned char raw[];
     __shared__ PlaneArgs sa;
@@ -364,12 +424,13 @@ __global__ void __launch_bounds__(LeanCfg<WY, HASMP>::kLT, HASMP ? 3 : 4)
         }
         sa = args[lo];
         sa.sweep += sweep_add;
+        sweep_key(sa.seed, sa.sweep, &sa.key);
         const int64_t local = blk - start[lo];
         s_zidx = (int)(local / sa.tiles);
         s_tile = (int)(local - (int64_t)s_zidx * sa.tiles);
     }
     __syncthreads();
-    lean_body<WY, FIELD, HASMP, false>(sa, nullptr, s_tile, s_zidx, raw);
+    lean_body<WY, FIELD, HASMP>(sa, nullptr, s_tile, s_zidx, raw);
 }
 
 PFN_cuTensorMapEncodeTiled_v12000 map_encoder() {
@@ -423,15 +484,16 @@ int lean_configure(size_t smem) {
 
 template <int WY, int FIELD, bool HASMP>
 int launch_lean(const PlaneArgs& a, int planes, cudaStream_t s) {
-    using Cfg = LeanCfg<WY, HASMP>;
+    using Cfg = LeanCfg<WY, FIELD, HASMP>;
     constexpr size_t smem = Cfg::smem();
     HP_CUDA_ONCE_ATTR(WY, FIELD, HASMP, smem);
     if (a.tiles == 0 || planes == 0) return HP_OK;
     LeanMaps maps;
     memset(&maps, 0, sizeof(maps));
     bool ok = a.Lx >= 64 && encode_box(&maps.q_in, a.q_in, a, WY) && encode_box(&maps.q_nb, a.q_nb, a, WY);
-    if (ok && HASMP) ok = encode_box(&maps.mp_in, a.mp_in, a, WY) && encode_box(&maps.mp_nb, a.mp_nb, a, WY);
+    if (ok && HASMP) ok = encode_box(&maps.mp_in, a.mp_in, a, WY);
     maps.ok = ok ? 1 : 0;
+    if (ok && HASMP) maps.pfm = encode_box(&maps.mp_nb, a.mp_nb, a, WY) ? 1 : 0;
     // a per-point field table of one entry per site shares the lattice's layout
     if (ok && FIELD == 2 && a.table_n == (uint32_t)((uint64_t)a.Lx * a.Ly * a.Lz) &&
         (uint64_t)a.Lx * a.Ly * a.Lz <= 0xFFFFFFFFull)
@@ -445,7 +507,7 @@ int launch_lean(const PlaneArgs& a, int planes, cudaStream_t s) {
 template <int WY, int FIELD, bool HASMP>
 int launch_lean_batch(const PlaneArgs* d_args, const int64_t* d_start, int R, int64_t blocks, uint32_t sweep_add,
                       cudaStream_t s) {
-    using Cfg = LeanCfg<WY, HASMP>;
+    using Cfg = LeanCfg<WY, FIELD, HASMP>;
     constexpr size_t smem = Cfg::smem();
     HP_CUDA_ONCE_ATTR(WY, FIELD, HASMP, smem);
     if (blocks == 0) return HP_OK;  // configure only (outside a graph capture)

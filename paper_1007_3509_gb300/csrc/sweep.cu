@@ -643,8 +643,8 @@ PlaneArgs plane_args(const hp_handle* h, int variant, const int32_t* q_in, const
     a.D = h->D;
     a.J = h->desc.J_fix;
     a.seed = h->desc.seed;
-    philox_round_keys(a.seed, a.rk);
     a.sweep = sweep;
+    sweep_key(a.seed, a.sweep, &a.key);
     a.Lx = (int)h->lat.L[0];
     a.Ly = (int)h->lat.L[1];
     a.Lz = (int)h->lat.L[2];
@@ -675,11 +675,11 @@ int plane_launch_batch(int nbr, int variant, int field, bool m, const PlaneArgs*
 
 // Variant a handle sweeps with until one is chosen (hp_set_sweep_variant or the
 // autotuner): the fastest measured on the benchmark lattices -- in 3D the lean
-// 64 x 32 window with material points (four blocks per SM) and the 64 x 44 one
-// without; in 2D the 128 x 60 lean tile.
+// 64 x 32 window (512^3, grain field: 1.25e11 site-updates/s against 1.03e11 of
+// 64 x 44); in 2D the 128 x 60 lean tile.
 int default_variant(const hp_handle* h) {
     int v = 0;
-    if (h->lat.nbr == 26) v = h->mp ? 11 : 8;
+    if (h->lat.nbr == 26) v = 11;
     else if (h->lat.nbr == 8 || h->lat.nbr == 4) v = 4;
     // variant 0 is built for every field mode; the others for the production ones
     return variant_ok(h->lat.nbr, v, h->desc.field_mode, h->mp != nullptr) ? v : 0;

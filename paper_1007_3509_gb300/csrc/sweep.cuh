@@ -29,7 +29,7 @@ struct PlaneArgs {
     int tiles;              // tiles per plane
     int fast;               // 1: window narrower than the lattice (wrap by one add)
     int vec;                // 1: fast and Lx % 4 == 0 (16-byte row chunks)
-    uint32_t rk[20];        // Philox round keys of seed (philox_round_keys)
+    SweepKey key;           // what the draws of (seed, sweep) share
 };
 
 namespace {
@@ -180,7 +180,7 @@ int tile_launch_batch(const PlaneArgs* d_args, const int64_t* d_start, int R, in
 int tile_status(int* timed_out);
 
 // Lean 3D kernel (lean.cu): one launch over the planes of one parity; 64 x WY
-// windows (WY 40 or 44), draws made while the window is in flight.
+// windows (WY 32, 36, 40 or 44), draws made while the window is in flight.
 int lean_launch(const PlaneArgs& a, int field, bool hasmp, int planes, int WY, cudaStream_t s);
 // The same over many lattices (see tile_launch_batch).
 int lean_launch_batch(const PlaneArgs* d_args, const int64_t* d_start, int R, int64_t blocks, uint32_t sweep_add,
