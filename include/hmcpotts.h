@@ -451,7 +451,7 @@ HP_API int hp_cp_step(const hp_cp_params* prm, uint64_t seed, const int32_t* gra
  * when the largest change of a strain component in one iteration is below
  * tol max|E| or after max_iter; *iters and *change (may be NULL) report the
  * iteration count and the last relative change.  FP32; allocates its work
- * buffer (six complex fields, 48 bytes per voxel) for the call; synchronous.
+ * buffer (six half spectra, 24 bytes per voxel) for the call; synchronous.
  * Voigt order xx yy zz yz xz xy, tensor components throughout.              */
 typedef struct {
     int32_t n[3];
