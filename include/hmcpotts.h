@@ -242,13 +242,15 @@ HP_API int hp_sweep(hp_handle* h, int32_t n_mcs, void* stream);
  * 26-neighbour lattice, lean 3D windows (64 x 44, 40, 36, 32: variants 8-11;
  * every random number drawn while the window is in flight).  Until a variant is
  * chosen, a handle sweeps with the fastest measured for its kind of lattice:
- * variant 11 in 3D, 4 in 2D.
+ * variant 11 in 3D, 3 or 4 in 2D; a small 2D lattice without material points is
+ * instead kept in the shared memory of a thread-block cluster for the whole call.
  * hp_sweep_variants: how many exist for `nbr`.
  * hp_set_sweep_variant: choose one (HP_ERR_ARG if not built for the handle's
  * field mode).  hp_sweep_autotune: time every variant for n_mcs MCS on a
  * backup of the bound state (the lattice and sweep counter are restored),
- * keep the fastest, write per-variant milliseconds to ms_out (host float[n],
- * -1 for unavailable variants; may be NULL) and the choice to *chosen.
+ * keep the fastest (or the resident 2D kernel, where the lattice takes it and it
+ * beats them all), write per-variant milliseconds to ms_out (host float[n], -1
+ * for unavailable variants; may be NULL) and the fastest variant to *chosen.
  * Allocates a temporary copy of the lattice; synchronises `stream`.          */
 HP_API int hp_sweep_variants(int32_t nbr, int32_t* n);
 HP_API int hp_set_sweep_variant(hp_handle* h, int32_t v);
@@ -373,16 +375,18 @@ HP_API int hp_ensemble_create(hp_handle* const* members, int32_t R, hp_ensemble*
 /* Free the ensemble's graph, capture stream and device argument arrays; the
  * members stay valid and belong to the caller.  Safe with NULL.              */
 HP_API int hp_ensemble_destroy(hp_ensemble* e);
-/* Tile variant used by hp_ensemble_sweep (default 0); HP_ERR_ARG for a variant
- * not built for the members' field mode.  Lean 3D windows of an ensemble are
- * filled by 16-byte asynchronous copies (no tiled TMA descriptors per member). */
+/* Tile variant used by hp_ensemble_sweep (until one is chosen, as for a handle:
+ * see hp_set_sweep_variant); HP_ERR_ARG for a variant not built for the members'
+ * field mode.  Lean 3D windows of an ensemble are filled by asynchronous copies
+ * (no tiled TMA descriptors per member).                                      */
 HP_API int hp_ensemble_set_variant(hp_ensemble* e, int32_t v);
 /* Pick the fastest tile variant for the whole ensemble (state restored).      */
 HP_API int hp_ensemble_autotune(hp_ensemble* e, int32_t n_mcs, float* ms_out, int32_t* chosen, void* stream);
 /* Sweep every member n_mcs MCS, bit-identical to hp_sweep on each member.  All
  * replicas share each launch (one CTA per replica tile); the n_mcs launches are
  * captured once into a CUDA graph (re-captured when n_mcs or the variant
- * changes) and replayed as one graph launch on `stream`.                      */
+ * changes) and replayed as one graph launch on `stream`.  Small 2D replicas whose
+ * tile variant was not chosen run resident instead, one cluster each.         */
 HP_API int hp_ensemble_sweep(hp_ensemble* e, int32_t n_mcs, void* stream);
 
 /* ------------------------------------------------------------------------ */

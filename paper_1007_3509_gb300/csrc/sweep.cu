@@ -676,13 +676,31 @@ int plane_launch_batch(int nbr, int variant, int field, bool m, const PlaneArgs*
 // Variant a handle sweeps with until one is chosen (hp_set_sweep_variant or the
 // autotuner): the fastest measured on the benchmark lattices -- in 3D the lean
 // 64 x 32 window (512^3, grain field: 1.25e11 site-updates/s against 1.03e11 of
-// 64 x 44); in 2D the 128 x 60 lean tile.
+// 64 x 44); in 2D the 128 x 28 lean tile (4 neighbours, 500^2 and 4096^2: 10.2 and
+// 61.6 us per MCS against 14.5 and 64.2 of 128 x 60; 8 neighbours, 1024^2: 12.7
+// against 16.8), but for 8 neighbours from 2048^2 sites on, where its halo costs
+// more than its latency saves, 128 x 60 (4096^2: 70.4 against 82.7).
 int default_variant(const hp_handle* h) {
     int v = 0;
     if (h->lat.nbr == 26) v = 11;
-    else if (h->lat.nbr == 8 || h->lat.nbr == 4) v = 4;
+    else if (h->lat.nbr == 4) v = 3;
+    else if (h->lat.nbr == 8) v = h->lat.N < (int64_t)1 << 22 ? 3 : 4;
     // variant 0 is built for every field mode; the others for the production ones
     return variant_ok(h->lat.nbr, v, h->desc.field_mode, h->mp != nullptr) ? v : 0;
+}
+
+// Cluster size when these lattices are better swept by the resident 2D kernel, else
+// 0.  One lattice: 8 SMs at 0.1 us per MCS and 1000 sites against the tile
+// kernel's floor of 10 to 12 us a launch (300^2: 9.9 us per MCS against 10.3 and
+// 12.1 for 4 and 8 neighbours; 500^2: 18 against 10 and 12).  Several: the same
+// size each, or enough of them to fill the chip (8 neighbours, kT = 1, 100 MCS:
+// 32 x 500^2 6.0 ms against 6.7, 100 x 500^2 14.0 against 19.5, but 4 x 500^2 2.0
+// against 1.6).
+int resident(hp_handle* const* m, int R) {
+    int64_t sites = 0;
+    for (int r = 0; r < R; ++r) sites += m[r]->lat.N;
+    const int cs = res2d_cluster(m, R);
+    return cs && (sites <= (int64_t)R * 100000 || (int64_t)R * cs >= 152) ? cs : 0;
 }
 
 int sweep_variants(int nbr) { return n_variants(nbr); }
@@ -703,6 +721,15 @@ int sweep_run(hp_handle* h, int32_t n_mcs, cudaStream_t s) {
             }
         h->sweep += (uint64_t)n_mcs;
         return HP_OK;
+    }
+    if (h->sweep_kernel == HP_SWEEP_AUTO && h->sweep_variant < 0) {
+        const int cs = resident(&h, 1);
+        if (cs) {
+            const int rc = res2d_run(&h, 1, cs, n_mcs, s);
+            if (rc) return rc;
+            h->sweep += (uint64_t)n_mcs;
+            return HP_OK;
+        }
     }
     const bool m = h->mp != nullptr;
     const int v = h->sweep_variant >= 0 ? h->sweep_variant : default_variant(h);
@@ -793,6 +820,18 @@ extern "C" int hp_sweep_autotune(hp_handle* h, int32_t n_mcs, float* ms_out, int
     h->sweep = sweep0;
     h->sweep_kernel = kernel0;
     h->sweep_variant = best;
+    // a lattice that the resident 2D kernel takes keeps to it when it beats them all
+    const int cs = rc == HP_OK && kernel0 == HP_SWEEP_AUTO ? resident(&h, 1) : 0;
+    if (cs && (rc = res2d_run(&h, 1, cs, 1, s)) == HP_OK) {
+        cudaEventRecord(e0, s);
+        rc = res2d_run(&h, 1, cs, n_mcs, s);
+        cudaEventRecord(e1, s);
+        float ms = 0.0f;
+        if (rc == HP_OK && cudaEventSynchronize(e1) == cudaSuccess && cudaEventElapsedTime(&ms, e0, e1) == cudaSuccess &&
+            ms < best_ms)
+            h->sweep_variant = -1;
+        cudaMemcpyAsync(h->q, bq, bytes, cudaMemcpyDeviceToDevice, s);
+    }
     cudaFreeAsync(bq, s);
     if (bm) cudaFreeAsync(bm, s);
     cudaEventDestroy(e0);
@@ -806,7 +845,7 @@ struct hp_ensemble {
     std::vector<hp_handle*> m;
     int nbr = 0, field = 0;
     bool hasmp = false;
-    int variant = 0;
+    int variant = -1;              // tile variant, -1 until one is chosen
     std::vector<PlaneArgs> args;   // [mcs parity][zpar][R]
     std::vector<int64_t> start;    // R + 1
     PlaneArgs* d_args = nullptr;
@@ -819,7 +858,10 @@ struct hp_ensemble {
 
 namespace {
 
+int ensemble_variant(const hp_ensemble* e) { return e->variant >= 0 ? e->variant : default_variant(e->m[0]); }
+
 int ensemble_build(hp_ensemble* e, cudaStream_t s) {
+    const int variant = ensemble_variant(e);
     const int R = (int)e->m.size();
     e->args.assign((size_t)4 * R, PlaneArgs{});
     e->start.assign((size_t)R + 1, 0);
@@ -832,9 +874,9 @@ int ensemble_build(hp_ensemble* e, cudaStream_t s) {
             int32_t* in_m = e->hasmp ? (k == 0 ? h->mp : h->mp_alt) : nullptr;
             int32_t* out_m = e->hasmp ? (k == 0 ? h->mp_alt : h->mp) : nullptr;
             e->args[(size_t)(2 * k + 0) * R + r] =
-                plane_args(h, e->variant, in_q, in_m, in_q, in_m, out_q, out_m, (uint32_t)h->sweep, 0, &planes);
+                plane_args(h, variant, in_q, in_m, in_q, in_m, out_q, out_m, (uint32_t)h->sweep, 0, &planes);
             e->args[(size_t)(2 * k + 1) * R + r] =
-                plane_args(h, e->variant, in_q, in_m, out_q, out_m, out_q, out_m, (uint32_t)h->sweep, 1, &planes);
+                plane_args(h, variant, in_q, in_m, out_q, out_m, out_q, out_m, (uint32_t)h->sweep, 1, &planes);
         }
         e->start[r + 1] = e->start[r] + (int64_t)e->args[r].tiles * planes;
     }
@@ -850,7 +892,7 @@ int ensemble_launches(hp_ensemble* e, int32_t n, cudaStream_t s, unsigned long l
     for (int32_t t = 0; t < n; ++t) {
         const int k = t & 1;
         for (int zp = 0; zp < (e->nbr == 26 ? 2 : 1); ++zp) {
-            const int rc = plane_launch_batch(e->nbr, e->variant, e->field, e->hasmp, e->d_args + (size_t)(2 * k + zp) * R,
+            const int rc = plane_launch_batch(e->nbr, ensemble_variant(e), e->field, e->hasmp, e->d_args + (size_t)(2 * k + zp) * R,
                                               e->d_start, R, blocks, (uint32_t)t, s);
             if (rc) return rc;
             ++nk;
@@ -947,12 +989,20 @@ extern "C" int hp_ensemble_sweep(hp_ensemble* e, int32_t n_mcs, void* stream) {
     if (!e || n_mcs < 0) return set_error(HP_ERR_ARG, "hp_ensemble_sweep: bad arguments");
     if (n_mcs == 0) return HP_OK;
     cudaStream_t s = as_stream(stream);
-    int rc = ensemble_build(e, s);  // refresh per-member sweep counters
+    int rc = HP_OK;
+    const int cs = e->variant < 0 ? resident(e->m.data(), (int)e->m.size()) : 0;
+    if (cs) {
+        if ((rc = res2d_run(e->m.data(), (int)e->m.size(), cs, n_mcs, s))) return rc;
+        for (hp_handle* h : e->m) h->sweep += (uint64_t)n_mcs;
+        return HP_OK;
+    }
+    rc = ensemble_build(e, s);  // refresh per-member sweep counters
     if (rc) return rc;
-    if (!e->exec || e->exec_n != n_mcs || e->exec_variant != e->variant) {
+    const int variant = ensemble_variant(e);
+    if (!e->exec || e->exec_n != n_mcs || e->exec_variant != variant) {
         if (e->exec) { cudaGraphExecDestroy(e->exec); e->exec = nullptr; }
         // kernel attributes are set outside the capture
-        rc = plane_launch_batch(e->nbr, e->variant, e->field, e->hasmp, e->d_args, e->d_start, 1, 0, 0, s);
+        rc = plane_launch_batch(e->nbr, variant, e->field, e->hasmp, e->d_args, e->d_start, 1, 0, 0, s);
         if (rc) return rc;
         cudaGraph_t g = nullptr;
         HP_CUDA(cudaStreamBeginCapture(e->cap, cudaStreamCaptureModeThreadLocal));
@@ -965,7 +1015,7 @@ extern "C" int hp_ensemble_sweep(hp_ensemble* e, int32_t n_mcs, void* stream) {
         cudaGraphDestroy(g);
         if (ie != cudaSuccess) { e->exec = nullptr; return cuda_error(ie, "hp_ensemble_sweep: instantiate"); }
         e->exec_n = n_mcs;
-        e->exec_variant = e->variant;
+        e->exec_variant = variant;
         e->exec_kernels = nk;
     } else {
         count_launch_n(e->exec_kernels);
@@ -1022,6 +1072,18 @@ extern "C" int hp_ensemble_autotune(hp_ensemble* e, int32_t n_mcs, float* ms_out
         restore();
     }
     e->variant = rc == HP_OK ? best : v0;
+    // members that the resident 2D kernel takes keep to it when it beats every variant
+    const int R = (int)e->m.size(), cs = rc == HP_OK ? resident(e->m.data(), R) : 0;
+    if (cs && (rc = res2d_run(e->m.data(), R, cs, 1, s)) == HP_OK) {
+        cudaEventRecord(e0, s);
+        rc = res2d_run(e->m.data(), R, cs, n_mcs, s);
+        cudaEventRecord(e1, s);
+        float ms = 0.0f;
+        if (rc == HP_OK && cudaEventSynchronize(e1) == cudaSuccess && cudaEventElapsedTime(&ms, e0, e1) == cudaSuccess &&
+            ms < best_ms)
+            e->variant = -1;
+        restore();
+    }
     for (size_t r = 0; r < e->m.size(); ++r) {
         if (bq[r]) cudaFreeAsync(bq[r], s);
         if (bm[r]) cudaFreeAsync(bm[r], s);
@@ -1029,7 +1091,7 @@ extern "C" int hp_ensemble_autotune(hp_ensemble* e, int32_t n_mcs, float* ms_out
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     if (cudaStreamSynchronize(s) != cudaSuccess && rc == HP_OK) rc = cuda_error(cudaGetLastError(), "hp_ensemble_autotune");
-    if (chosen) *chosen = e->variant;
+    if (chosen) *chosen = best;
     return rc;
 }
 

@@ -188,5 +188,12 @@ int lean_launch_batch(const PlaneArgs* d_args, const int64_t* d_start, int R, in
 // Reads and clears the lean kernel's timeout flag (2: a drain ran out too).
 int lean_status(int* timed_out);
 
+// Resident 2D sweep (res2d.cu): cluster size for these lattices (all of one dim, nbr,
+// field mode), 0 when one of them does not fit or is of another kind.
+int res2d_cluster(hp_handle* const* m, int R);
+// n_mcs MCS of every lattice, in place, from each handle's sweep counter (not
+// advanced here).
+int res2d_run(hp_handle* const* m, int R, int cs, int32_t n_mcs, cudaStream_t s);
+
 
 }  // namespace hp

@@ -87,8 +87,8 @@ struct Tile {
     __device__ __forceinline__ bool draw_site(uint32_t e, uint32_t colour, uint2& w) const {
         const int r = (int)(e >> 8), col = (int)(e & 255u);
         const int pos = r * WX + col;
-        const uint4 u = draw(a.seed, (uint64_t)(gx_of(col) + (int64_t)a.Lx * gy_of(r) + sxy * z), a.sweep, kTagSweep,
-                             colour);
+        const uint2 u = sweep_draw(a.key, (uint32_t)gx_of(col) + (uint32_t)a.Lx * (uint32_t)gy_of(r) +
+                                              (uint32_t)sxy * (uint32_t)z, colour);
         const int kp = (int)__umulhi(u.x, (uint32_t)M);
         int dx, dy, dz;
         offs(kp, dx, dy, dz);
@@ -369,6 +369,7 @@ __global__ void __launch_bounds__(kTileThreads, NBR == 26 ? 4 : 5)
         }
         sa = args[lo];
         sa.sweep += sweep_add;
+        sweep_key(sa.seed, sa.sweep, &sa.key);
         const int64_t local = blk - start[lo];
         s_zidx = (int)(local / sa.tiles);
         s_tile = (int)(local - (int64_t)s_zidx * sa.tiles);
