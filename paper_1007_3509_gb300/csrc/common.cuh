@@ -114,6 +114,22 @@ __device__ __forceinline__ uint4 draw(uint64_t seed, uint64_t unit, uint32_t ste
                      make_uint4((uint32_t)unit, (uint32_t)(unit >> 32), step, (tag << 24) | sub));
 }
 
+// The four cubic invariants of the loading axis d = R(q)^T e_x that the surrogate
+// sees: |d| sorted in decreasing order and d1^2 d2^2 + d2^2 d3^2 + d3^2 d1^2.
+__device__ __forceinline__ void orient_features(const float* q, float* f) {
+    const float n = rsqrtf(q[0] * q[0] + q[1] * q[1] + q[2] * q[2] + q[3] * q[3]);
+    const float w = q[0] * n, x = q[1] * n, y = q[2] * n, z = q[3] * n;
+    float a = fabsf(1.0f - 2.0f * (y * y + z * z)), b = fabsf(2.0f * (x * y - w * z)), c = fabsf(2.0f * (x * z + w * y));
+    float t;
+    if (a < b) { t = a; a = b; b = t; }
+    if (b < c) { t = b; b = c; c = t; }
+    if (a < b) { t = a; a = b; b = t; }
+    f[0] = a;
+    f[1] = b;
+    f[2] = c;
+    f[3] = a * a * b * b + b * b * c * c + c * c * a * a;
+}
+
 // ---------------------------------------------------------------------------
 // Handle
 // ---------------------------------------------------------------------------
@@ -165,6 +181,18 @@ int orientations_run(int32_t G, uint64_t seed, int32_t kind, float* orient, cuda
 // raised exactly as by a kernel that timed out.
 int lean_wait_probe(long long limit, int late, cudaStream_t s);
 int mlp_wait_probe(long long limit, int late, cudaStream_t s);
+
+// The per-grain field of hp_sur_field in one launch: features of quat[4 G] and the
+// load state in, quantised energies b (and e, may be null) out.
+struct FieldIO {
+    const float* quat;
+    float load[7];                     // stress[6], slip
+    float stress, strain, w, erho;     // hp_sur_scales
+    float scale;                       // energy_scale
+    int32_t* b;
+    float* e;
+};
+int mlp_field(const float* params, const FieldIO& io, int32_t G, cudaStream_t s);
 
 // Training state of one hp_sur_train call: the packed weight image and the
 // per-CTA gradient slots, owned by the call.

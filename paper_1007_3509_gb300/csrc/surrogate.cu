@@ -87,20 +87,6 @@ struct Scales {
     float stress, strain, w, erho;
 };
 
-__device__ __forceinline__ void orient_features(const float* q, float* f) {
-    const float n = rsqrtf(q[0] * q[0] + q[1] * q[1] + q[2] * q[2] + q[3] * q[3]);
-    const float w = q[0] * n, x = q[1] * n, y = q[2] * n, z = q[3] * n;
-    float a = fabsf(1.0f - 2.0f * (y * y + z * z)), b = fabsf(2.0f * (x * y - w * z)), c = fabsf(2.0f * (x * z + w * y));
-    float t;
-    if (a < b) { t = a; a = b; b = t; }
-    if (b < c) { t = b; b = c; c = t; }
-    if (a < b) { t = a; a = b; b = t; }
-    f[0] = a;
-    f[1] = b;
-    f[2] = c;
-    f[3] = a * a * b * b + b * b * c * c + c * c * a * a;
-}
-
 // Writes row o * row_stride of X and Y (row_stride = n_incr, X and Y offset to the increment).
 __global__ void k_collect(int32_t n_orient, int32_t K, const float* quat, const float* w, const float* erho,
                           const double* acc, double inv_p, Scales sc, int32_t row_stride, float* X, float* Y) {
@@ -123,31 +109,6 @@ __global__ void k_collect(int32_t n_orient, int32_t K, const float* quat, const 
 
 __global__ void k_load_out(const double* acc, double inv_p, float* out) {
     if (threadIdx.x < 7) out[threadIdx.x] = (float)(acc[threadIdx.x] * inv_p);
-}
-
-// the load state of the current increment, passed by value
-struct Load7 {
-    float v[7];
-};
-
-__global__ void k_field_inputs(int32_t G, const float* quat, const Load7 load, Scales sc, float* X) {
-    const int32_t g = blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= G) return;
-    float* x = X + (int64_t)g * 11;
-    orient_features(quat + 4 * (int64_t)g, x);
-#pragma unroll
-    for (int c = 0; c < 6; ++c) x[4 + c] = load.v[c] / sc.stress;
-    x[10] = load.v[6] / sc.strain;
-}
-
-__global__ void k_field_quantise(int32_t G, const float* Y, Scales sc, float energy_scale, int32_t* b, float* e_out) {
-    const int32_t g = blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= G) return;
-    const float e = energy_scale * (Y[2 * (int64_t)g] * sc.w + Y[2 * (int64_t)g + 1] * sc.erho);
-    if (e_out) e_out[g] = e;
-    float v = rintf(256.0f * e);
-    v = fminf(fmaxf(v, -1048576.0f), 1048576.0f);
-    b[g] = (int32_t)v;
 }
 
 }  // namespace
@@ -211,29 +172,17 @@ extern "C" int hp_sur_generate(const hp_cp_params* prm, uint64_t seed, const flo
 extern "C" int hp_sur_field(const float* params, const float* quat, int32_t G, const float* load,
                             const hp_sur_scales* sc, double energy_scale, int32_t* b_out, float* e_out, void* stream) {
     if (!params || !quat || G < 1 || !load || !sc || !b_out) return set_error(HP_ERR_ARG, "hp_sur_field: bad arguments");
-    cudaStream_t s = as_stream(stream);
-    float *X = nullptr, *Y = nullptr;
-    if (cudaMallocAsync((void**)&X, sizeof(float) * 11 * (size_t)G, s) != cudaSuccess ||
-        cudaMallocAsync((void**)&Y, sizeof(float) * 2 * (size_t)G, s) != cudaSuccess) {
-        cudaFreeAsync(X, s); cudaFreeAsync(Y, s);
-        return set_error(HP_ERR_OOM, "hp_sur_field: allocation failed");
-    }
-    Scales scl{sc->stress, sc->strain, sc->w, sc->erho};
-    Load7 lv;
-    for (int c = 0; c < 7; ++c) lv.v[c] = load[c];  // copied into the launch: the caller may free load
-    ::hp::count_launch();
-    k_field_inputs<<<(G + kT - 1) / kT, kT, 0, s>>>(G, quat, lv, scl, X);
-    cudaError_t e = cudaGetLastError();
-    int rc = e == cudaSuccess ? hp_mlp_forward(params, X, G, Y, stream) : HP_OK;
-    if (e == cudaSuccess && rc == HP_OK) {
-        ::hp::count_launch();
-        k_field_quantise<<<(G + kT - 1) / kT, kT, 0, s>>>(G, Y, scl, (float)energy_scale, b_out, e_out);
-        e = cudaGetLastError();
-    }
-    if (e != cudaSuccess && rc == HP_OK) rc = cuda_error(e, "hp_sur_field");
-    cudaFreeAsync(X, s);
-    cudaFreeAsync(Y, s);
-    return rc;
+    FieldIO io;
+    io.quat = quat;
+    for (int c = 0; c < 7; ++c) io.load[c] = load[c];  // copied into the launch: the caller may free load
+    io.stress = sc->stress;
+    io.strain = sc->strain;
+    io.w = sc->w;
+    io.erho = sc->erho;
+    io.scale = (float)energy_scale;
+    io.b = b_out;
+    io.e = e_out;
+    return mlp_field(params, io, G, as_stream(stream));
 }
 
 extern "C" int hp_sur_train(float* params, float* m, float* v, const float* X, const float* Y, int64_t M,
