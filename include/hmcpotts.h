@@ -168,9 +168,10 @@ HP_API int hp_set_field(hp_handle* h, const int32_t* table, int64_t n);
  * trial is scaled by the mobility m of the (q_i, q_j) boundary: eff = thr[d]
  * (0xFFFFFFFF for d < 0) if m is 0xFFFFFFFF, m if thr[d] is, else
  * floor(thr[d] m / 2^32); accept iff d <= D and (eff == 0xFFFFFFFF or u1 < eff).
- * With tables set, hp_sweep runs the per-colour kernel; angle = J = NULL
- * clears them (back to the constant J_fix).  Copies the tables; synchronises
- * `stream`.                                                                  */
+ * With tables set, hp_sweep takes a kernel built for them (2D lattices: fused
+ * tiles, whatever variant is chosen; others and HP_SWEEP_PHASE: per colour);
+ * angle = J = NULL clears them (back to the constant J_fix).  Copies the tables;
+ * synchronises `stream`.                                                     */
 HP_API int hp_set_anisotropy(hp_handle* h, const int32_t* angle, int32_t period, int32_t bin, int32_t nbins,
                              const int32_t* J, const uint32_t* mobility, void* stream);
 

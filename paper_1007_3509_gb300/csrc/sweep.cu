@@ -40,26 +40,10 @@ struct PhaseArgs {
     uint32_t sweep;
     int colour;
     int Lx, Ly, Lz;
-    int64_t n_colour_sites;
-    // misorientation-dependent pair energy and mobility (ANI kernels only)
-    const int32_t* ang;   // grain angles (borrowed, G entries)
-    const int32_t* jtab;  // energy per misorientation bin (256 = 1 J)
-    const uint32_t* mob;  // relative mobility per bin (all ones = 1), or null
-    int32_t period, bin_w, nbins, G;
+    uint32_t n_colour_sites;
+    SweepKey key;
+    Aniso an;             // misorientation-dependent pair energy and mobility (ANI kernels only)
 };
-
-// Misorientation bin of grains a and b: |ang_a - ang_b| folded by the angle's
-// symmetry period, divided by the bin width, clamped to the last bin (grain ids
-// clamped into the table: they come from caller buffers).
-__device__ __forceinline__ int mis_bin(const PhaseArgs& a, int32_t qa, int32_t qb) {
-    const uint32_t ua = (uint32_t)qa < (uint32_t)a.G ? (uint32_t)qa : (uint32_t)(a.G - 1);
-    const uint32_t ub = (uint32_t)qb < (uint32_t)a.G ? (uint32_t)qb : (uint32_t)(a.G - 1);
-    int64_t d = (int64_t)__ldg(a.ang + ua) - (int64_t)__ldg(a.ang + ub);
-    d = (d < 0 ? -d : d) % a.period;
-    if (a.period - d < d) d = a.period - d;
-    const int64_t k = d / a.bin_w;
-    return (int)(k < a.nbins ? k : a.nbins - 1);
-}
 
 // ---------------------------------------------------------------------------
 // One colour phase, one thread per site of that colour, in place.
@@ -67,87 +51,88 @@ __device__ __forceinline__ int mis_bin(const PhaseArgs& a, int32_t qa, int32_t q
 // ---------------------------------------------------------------------------
 // ANI: the energy of a site in state s is the sum over neighbours n with
 // q_n != s of jtab[bin(s, q_n)], and the Metropolis threshold is scaled by the
-// mobility of the (q_i, q_j) boundary: eff = thr[d] (all ones for d < 0) when
-// the mobility m is all ones, m when thr is all ones, else floor(thr m / 2^32);
-// accept iff d <= D and (eff is all ones or u1 < eff).
+// mobility of the (q_i, q_j) boundary (metropolis_mob).
 template <int DIM, int NBR, int FIELD, bool HASMP, bool ANI>
-__global__ void __launch_bounds__(kThreads) k_phase(PhaseArgs a) {
+__global__ void __launch_bounds__(kThreads) k_phase(const __grid_constant__ PhaseArgs a) {
     using G = Geo<DIM, NBR>;
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;  // lattices hold fewer than 2^31 sites
     if (t >= a.n_colour_sites) return;
     const int c = a.colour;
-    const int hx = a.Lx >> 1;
+    const uint32_t hx = (uint32_t)a.Lx >> 1, r = t / hx;
+    const int xs = (int)(t - r * hx);
     int x, y, z;
     if (G::C == 2) {
-        const int64_t r = t / hx;
-        const int k = (int)(t - r * hx);
-        y = (int)(r % a.Ly);
-        z = (int)(r / a.Ly);
-        x = 2 * k + ((y + z + c) & 1);
+        z = DIM == 3 ? (int)(r / (uint32_t)a.Ly) : 0;
+        y = (int)(r - (uint32_t)z * (uint32_t)a.Ly);
+        x = 2 * xs + ((y + z + c) & 1);
     } else if (G::C == 4) {
-        const int64_t r = t / hx;
-        x = 2 * (int)(t - r * hx) + (c & 1);
+        x = 2 * xs + (c & 1);
         y = 2 * (int)r + (c >> 1);
         z = 0;
     } else {
-        const int hy = a.Ly >> 1;
-        const int64_t r = t / hx;
-        x = 2 * (int)(t - r * hx) + (c & 1);
-        y = 2 * (int)(r % hy) + ((c >> 1) & 1);
-        z = 2 * (int)(r / hy) + (c >> 2);
+        const uint32_t hy = (uint32_t)a.Ly >> 1, zs = r / hy;
+        x = 2 * xs + (c & 1);
+        y = 2 * (int)(r - zs * hy) + ((c >> 1) & 1);
+        z = 2 * (int)zs + (c >> 2);
     }
-    const int64_t sxy = (int64_t)a.Lx * a.Ly;
-    const int64_t i = x + (int64_t)a.Lx * y + sxy * z;
+    const uint32_t sxy = (uint32_t)a.Lx * (uint32_t)a.Ly;
+    const uint32_t i = (uint32_t)x + (uint32_t)a.Lx * (uint32_t)y + sxy * (uint32_t)z;
+    // columns, row and plane offsets of the neighbourhood, each wrapped once
+    uint32_t xc[3], yc[3], zc[3];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        xc[d] = (uint32_t)wrap1(x + d - 1, a.Lx);
+        yc[d] = (uint32_t)a.Lx * (uint32_t)wrap1(y + d - 1, a.Ly);
+        zc[d] = DIM == 3 ? sxy * (uint32_t)wrap1(z + d - 1, a.Lz) : 0u;
+    }
     const int32_t qi = a.q[i];
     int32_t nv[G::M];
-    int64_t ni[G::M];
     int same_old = 0;
 #pragma unroll
     for (int k = 0; k < G::M; ++k) {
         int dx, dy, dz;
         G::off(k, dx, dy, dz);
-        const int xx = wrapi(x + dx, a.Lx), yy = wrapi(y + dy, a.Ly), zz = DIM == 3 ? wrapi(z + dz, a.Lz) : 0;
-        ni[k] = xx + (int64_t)a.Lx * yy + sxy * zz;
-        nv[k] = a.q[ni[k]];
+        nv[k] = a.q[xc[dx + 1] + yc[dy + 1] + zc[dz + 1]];
         same_old += nv[k] == qi;
     }
     if (same_old == G::M) return;
-    const uint4 u = draw(a.seed, (uint64_t)i, a.sweep, kTagSweep, (uint32_t)c);
+    const uint2 u = sweep_draw(a.key, i, (uint32_t)c);
     const int kp = (int)__umulhi(u.x, (uint32_t)G::M);
     int32_t qj = 0;
-    int64_t j = 0;
+    uint32_t j = 0;
 #pragma unroll
-    for (int k = 0; k < G::M; ++k)
-        if (k == kp) { qj = nv[k]; j = ni[k]; }
+    for (int k = 0; k < G::M; ++k) {
+        int dx, dy, dz;
+        G::off(k, dx, dy, dz);
+        if (k == kp) {
+            qj = nv[k];
+            if (HASMP) j = xc[dx + 1] + yc[dy + 1] + zc[dz + 1];
+        }
+    }
     if (qj == qi) return;
-    int same_new = 0;
-#pragma unroll
-    for (int k = 0; k < G::M; ++k) same_new += nv[k] == qj;
     int32_t db = 0;
     int32_t mpj = 0;
     if (HASMP) mpj = a.mp[j];
     if (FIELD == 1) db = tab(a.table, a.table_n, qj) - tab(a.table, a.table_n, qi);
     if (FIELD == 2) db = tab(a.table, a.table_n, mpj) - tab(a.table, a.table_n, a.mp[i]);
+    bool flip;
     if (!ANI) {
-        const int32_t d = a.J * (same_old - same_new) + db;
-        if (metropolis(d, a.D, a.thr, u.y)) {
-            a.q[i] = qj;
-            if (HASMP) a.mp[i] = mpj;
-        }
-        return;
-    }
-    int32_t e_old = 0, e_new = 0;
+        int same_new = 0;
 #pragma unroll
-    for (int k = 0; k < G::M; ++k) {
-        if (nv[k] != qi) e_old += __ldg(a.jtab + mis_bin(a, qi, nv[k]));
-        if (nv[k] != qj) e_new += __ldg(a.jtab + mis_bin(a, qj, nv[k]));
+        for (int k = 0; k < G::M; ++k) same_new += nv[k] == qj;
+        flip = metropolis(a.J * (same_old - same_new) + db, a.D, a.thr, u.y);
+    } else {
+        const int32_t ai = mis_angle(a.an, qi), aj = mis_angle(a.an, qj);
+        int32_t e = db;
+#pragma unroll
+        for (int k = 0; k < G::M; ++k) {
+            const int32_t an = mis_angle(a.an, nv[k]);
+            if (nv[k] != qi) e -= __ldg(a.an.jtab + mis_bin(a.an, ai, an));
+            if (nv[k] != qj) e += __ldg(a.an.jtab + mis_bin(a.an, aj, an));
+        }
+        flip = metropolis_mob(a.an, e, a.D, a.thr, u.y, ai, aj);
     }
-    const int32_t d = e_new - e_old + db;
-    if (d > a.D) return;
-    const uint32_t th = d < 0 ? 0xFFFFFFFFu : __ldg(a.thr + d);
-    const uint32_t m = a.mob ? __ldg(a.mob + mis_bin(a, qi, qj)) : 0xFFFFFFFFu;
-    const uint32_t eff = m == 0xFFFFFFFFu ? th : (th == 0xFFFFFFFFu ? m : __umulhi(th, m));
-    if (eff == 0xFFFFFFFFu || u.y < eff) {
+    if (flip) {
         a.q[i] = qj;
         if (HASMP) a.mp[i] = mpj;
     }
@@ -472,19 +457,14 @@ int launch_phase(hp_handle* h, uint32_t sweep, int colour, cudaStream_t s) {
     a.J = h->desc.J_fix;
     a.seed = h->desc.seed;
     a.sweep = sweep;
+    sweep_key(a.seed, sweep, &a.key);
     a.colour = colour;
     a.Lx = (int)h->lat.L[0];
     a.Ly = (int)h->lat.L[1];
     a.Lz = (int)h->lat.L[2];
-    a.n_colour_sites = h->lat.N / Geo<DIM, NBR>::C;
-    a.ang = h->an_ang;
-    a.jtab = h->an_J;
-    a.mob = h->an_mob;
-    a.period = h->an_period;
-    a.bin_w = h->an_bin;
-    a.nbins = h->an_nbins;
-    a.G = h->desc.n_grains;
-    const int64_t blocks = (a.n_colour_sites + kThreads - 1) / kThreads;
+    a.n_colour_sites = (uint32_t)(h->lat.N / Geo<DIM, NBR>::C);
+    a.an = aniso_of(h);
+    const int64_t blocks = ((int64_t)a.n_colour_sites + kThreads - 1) / kThreads;
     ::hp::count_launch();
     k_phase<DIM, NBR, FIELD, HASMP, ANI><<<(unsigned)blocks, kThreads, 0, s>>>(a);
     HP_LAUNCH_CHECK("k_phase");
@@ -626,6 +606,8 @@ bool variant_batch_ok(int nbr, int v, int field, bool m) {
     return variant_ok(nbr, v, field, m);
 }
 
+constexpr int kAnisoVariant = 3;  // 128 x 28 lean tiles (the shape of tile_launch_aniso)
+
 // Arguments of the fused kernel for one lattice and one launch.
 PlaneArgs plane_args(const hp_handle* h, int variant, const int32_t* q_in, const int32_t* mp_in,
                      const int32_t* q_nb, const int32_t* mp_nb, int32_t* q_out, int32_t* mp_out, uint32_t sweep,
@@ -711,8 +693,11 @@ bool sweep_variant_batch_ok(int nbr, int v, int field, bool m) { return variant_
 
 int sweep_run(hp_handle* h, int32_t n_mcs, cudaStream_t s) {
     const int nbr = h->lat.nbr;
-    const bool fused_ok = nbr != 6 && !h->an_J;  // the pair-energy tables run on the per-colour kernel
-    const bool fused = fused_ok && h->sweep_kernel != HP_SWEEP_PHASE;
+    // with pair-energy tables 2D lattices run on the fused tiles where these are
+    // built, the others on the per-colour kernel
+    const bool tiles = h->an_J && h->lat.dim == 2 &&
+                       (h->mp ? h->desc.field_mode == HP_FIELD_POINT : h->desc.field_mode != HP_FIELD_POINT);
+    const bool fused = nbr != 6 && (!h->an_J || tiles) && h->sweep_kernel != HP_SWEEP_PHASE;
     if (!fused) {
         for (int32_t t = 0; t < n_mcs; ++t)
             for (int c = 0; c < h->lat.colours; ++c) {
@@ -732,7 +717,7 @@ int sweep_run(hp_handle* h, int32_t n_mcs, cudaStream_t s) {
         }
     }
     const bool m = h->mp != nullptr;
-    const int v = h->sweep_variant >= 0 ? h->sweep_variant : default_variant(h);
+    const int v = h->an_J ? kAnisoVariant : h->sweep_variant >= 0 ? h->sweep_variant : default_variant(h);
     int32_t *qc = h->q, *mc = h->mp, *qa = h->q_alt, *ma = m ? h->mp_alt : nullptr;
     for (int32_t t = 0; t < n_mcs; ++t) {
         Range r_("mcs");
@@ -746,7 +731,7 @@ int sweep_run(hp_handle* h, int32_t n_mcs, cudaStream_t s) {
             rc = plane_launch(h, v, a1, planes, s);
         } else {
             const PlaneArgs a0 = plane_args(h, v, qc, mc, nullptr, nullptr, qa, ma, sw, 0, &planes);
-            rc = plane_launch(h, v, a0, planes, s);
+            rc = h->an_J ? tile_launch_aniso(a0, aniso_of(h), h->desc.field_mode, m, nbr, s) : plane_launch(h, v, a0, planes, s);
         }
         if (rc) return rc;
         int32_t* tq = qc; qc = qa; qa = tq;

@@ -32,7 +32,56 @@ struct PlaneArgs {
     SweepKey key;           // what the draws of (seed, sweep) share
 };
 
+// Misorientation tables of hp_set_anisotropy: bin of grains a and b = |ang_a -
+// ang_b| folded by the angle's symmetry period, divided by the bin width, clamped
+// to the last bin.  The division is a multiplication (Granlund and Montgomery,
+// "Division by invariant integers using multiplication", 1994): floor(d / bin) =
+// (t + ((d - t) >> 1)) >> shift, t = mul d / 2^32, for every 32-bit d.
+struct Aniso {
+    const int32_t* ang;   // grain angles (borrowed, G entries)
+    const int32_t* jtab;  // energy per misorientation bin (256 = 1 J)
+    const uint32_t* mob;  // relative mobility per bin (all ones = 1), or null
+    uint32_t period, bin, mul, shift, last_bin, last_grain;
+};
+inline Aniso aniso_of(const hp_handle* h) {
+    Aniso a;
+    a.ang = h->an_ang;
+    a.jtab = h->an_J;
+    a.mob = h->an_mob;
+    a.period = (uint32_t)h->an_period;
+    a.bin = (uint32_t)h->an_bin;
+    a.last_bin = (uint32_t)h->an_nbins - 1u;
+    a.last_grain = (uint32_t)h->desc.n_grains - 1u;
+    uint32_t l = 0;
+    while (l < 32 && ((uint64_t)1 << l) < a.bin) ++l;
+    a.mul = a.bin ? (uint32_t)(((((uint64_t)1 << l) - a.bin) << 32) / a.bin + 1) : 0u;
+    a.shift = l ? l - 1 : 0;
+    return a;
+}
+
 namespace {
+
+// a grain's angle (the id clamped into the table: it comes from a caller buffer)
+__device__ __forceinline__ int32_t mis_angle(const Aniso& a, int32_t q) { return __ldg(a.ang + min((uint32_t)q, a.last_grain)); }
+__device__ __forceinline__ uint32_t mis_bin(const Aniso& a, int32_t ua, int32_t ub) {
+    uint32_t d = ua > ub ? (uint32_t)ua - (uint32_t)ub : (uint32_t)ub - (uint32_t)ua;
+    if (d >= a.period) d %= a.period;  // angles outside [0, period)
+    d = min(d, a.period - d);
+    const uint32_t t = __umulhi(a.mul, d);
+    const uint32_t k = a.bin == 1u ? d : (t + ((d - t) >> 1)) >> a.shift;
+    return min(k, a.last_bin);
+}
+// Trial with the mobility of the (q_i, q_j) boundary: eff = thr[d] (all ones for d <
+// 0) when the mobility m is all ones, m when thr is all ones, else floor(thr m /
+// 2^32); accept iff d <= D and (eff is all ones or u < eff).
+__device__ __forceinline__ bool metropolis_mob(const Aniso& an, int32_t d, int32_t D, const uint32_t* __restrict__ thr,
+                                               uint32_t u, int32_t ai, int32_t aj) {
+    if (d > D) return false;
+    const uint32_t th = d < 0 ? 0xFFFFFFFFu : __ldg(thr + d);
+    const uint32_t m = an.mob ? __ldg(an.mob + mis_bin(an, ai, aj)) : 0xFFFFFFFFu;
+    const uint32_t eff = m == 0xFFFFFFFFu ? th : (th == 0xFFFFFFFFu ? m : __umulhi(th, m));
+    return eff == 0xFFFFFFFFu || u < eff;
+}
 
 template <int DIM, int NBR>
 struct Geo;
@@ -176,6 +225,8 @@ int tile_launch(const PlaneArgs& a, int field, bool hasmp, int nbr, int planes, 
 // blocks == 0 only configures the kernel (outside a graph capture).
 int tile_launch_batch(const PlaneArgs* d_args, const int64_t* d_start, int R, int64_t blocks, uint32_t sweep_add,
                       int field, bool hasmp, int nbr, int WX, int WY, cudaStream_t s);
+// One launch over a 2D lattice with misorientation tables (128 x 32 windows).
+int tile_launch_aniso(const PlaneArgs& a, const Aniso& an, int field, bool hasmp, int nbr, cudaStream_t s);
 // Reads and clears the tile kernel's timeout flag.
 int tile_status(int* timed_out);
 

@@ -55,8 +55,9 @@ struct TileCfg {
     static size_t smem() { return 128 + sizeof(int32_t) * ((size_t)ARR * AS + QCAP + 8) + sizeof(uint2) * 64 * (kTileThreads / 32); }
 };
 
-template <int NBR, int WX, int WY, int FIELD, bool HASMP>
+template <int NBR, int WX, int WY, int FIELD, bool HASMP, bool ANI>
 struct Tile {
+    const Aniso* an;
     using Cfg = TileCfg<NBR, WX, WY, HASMP>;
     static constexpr int M = NBR;
     const PlaneArgs& a;
@@ -117,6 +118,23 @@ struct Tile {
         }
         if (FIELD == 1) { bi = tab(a.table, a.table_n, qi); bj = tab(a.table, a.table_n, qj); }
         if (FIELD == 2) { bi = tab(a.table, a.table_n, SMP[pos]); bj = tab(a.table, a.table_n, mpj); }
+        if (ANI) {  // 2D: pair energies and mobility by misorientation
+            const int32_t* c = S + pos;
+            const int32_t ai = mis_angle(*an, qi), aj = mis_angle(*an, qj);
+            int32_t e = bj - bi;
+            auto add = [&](int32_t v) {
+                const int32_t av = mis_angle(*an, v);
+                if (v != qi) e -= __ldg(an->jtab + mis_bin(*an, ai, av));
+                if (v != qj) e += __ldg(an->jtab + mis_bin(*an, aj, av));
+            };
+            add(c[-1]); add(c[1]); add(c[-WX]); add(c[WX]);
+            if (NBR == 8) { add(c[-WX - 1]); add(c[-WX + 1]); add(c[WX - 1]); add(c[WX + 1]); }
+            if (metropolis_mob(*an, e, a.D, a.thr, w.y, ai, aj)) {
+                S[pos] = qj;
+                if (HASMP) SMP[pos] = mpj;
+            }
+            return;
+        }
         int so = 0, sn = 0;
         auto cnt = [&](int32_t v) { so += v == qi; sn += v == qj; };
         const int32_t* c = S + pos;
@@ -150,9 +168,10 @@ struct Tile {
 
 __device__ __forceinline__ bool al16(const void* p) { return ((uintptr_t)p & 15u) == 0; }
 
-template <int NBR, int WX, int WY, int FIELD, bool HASMP>
-__device__ __forceinline__ void tile_body(const PlaneArgs& a, const int tile, const int zidx, unsigned char* raw) {
-    using T = Tile<NBR, WX, WY, FIELD, HASMP>;
+template <int NBR, int WX, int WY, int FIELD, bool HASMP, bool ANI>
+__device__ __forceinline__ void tile_body(const PlaneArgs& a, const int tile, const int zidx, unsigned char* raw,
+                                          const Aniso* an) {
+    using T = Tile<NBR, WX, WY, FIELD, HASMP, ANI>;
     using Cfg = typename T::Cfg;
     constexpr int ARR = Cfg::ARR, AS = Cfg::AS, PAD = Cfg::PAD, NP = Cfg::NP, QPR = Cfg::QPR;
     constexpr int M = NBR;
@@ -167,6 +186,7 @@ __device__ __forceinline__ void tile_body(const PlaneArgs& a, const int tile, co
     uint2* wqueue = reinterpret_cast<uint2*>(qn + 8);                          // 64 per warp
 
     T t(a);
+    t.an = an;
     t.S = base + PAD;
     t.SMP = base + (HASMP ? AS + PAD : PAD);
     t.SLO = base + Cfg::A_LO * AS + PAD;
@@ -349,7 +369,14 @@ __device__ __forceinline__ void tile_body(const PlaneArgs& a, const int tile, co
 template <int NBR, int WX, int WY, int FIELD, bool HASMP>
 __global__ void __launch_bounds__(kTileThreads, NBR == 26 ? 4 : 5) k_tile(const __grid_constant__ PlaneArgs a) {
     extern __shared__ __align__(16) unsigned char raw[];
-    tile_body<NBR, WX, WY, FIELD, HASMP>(a, (int)blockIdx.x, (int)blockIdx.y, raw);
+    tile_body<NBR, WX, WY, FIELD, HASMP, false>(a, (int)blockIdx.x, (int)blockIdx.y, raw, nullptr);
+}
+
+template <int NBR, int WX, int WY, int FIELD, bool HASMP>
+__global__ void __launch_bounds__(kTileThreads, 5)
+    k_tile_aniso(const __grid_constant__ PlaneArgs a, const __grid_constant__ Aniso an) {
+    extern __shared__ __align__(16) unsigned char raw[];
+    tile_body<NBR, WX, WY, FIELD, HASMP, true>(a, (int)blockIdx.x, 0, raw, &an);
 }
 
 // Many independent lattices in one launch: block b belongs to the replica r
@@ -375,7 +402,7 @@ __global__ void __launch_bounds__(kTileThreads, NBR == 26 ? 4 : 5)
         s_tile = (int)(local - (int64_t)s_zidx * sa.tiles);
     }
     __syncthreads();
-    tile_body<NBR, WX, WY, FIELD, HASMP>(sa, s_tile, s_zidx, raw);
+    tile_body<NBR, WX, WY, FIELD, HASMP, false>(sa, s_tile, s_zidx, raw, nullptr);
 }
 
 struct TileBatch {
@@ -438,7 +465,27 @@ int tile_dispatch(const PlaneArgs* a, const TileBatch* b, int field, bool hasmp,
     return set_error(HP_ERR_ARG, "sweep: no tile kernel of this shape");
 }
 
+template <int NBR, int FIELD, bool HASMP>
+int launch_aniso(const PlaneArgs& a, const Aniso& an, cudaStream_t s) {
+    const size_t smem = TileCfg<NBR, 128, 32, HASMP>::smem();
+    HP_CUDA(cudaFuncSetAttribute(k_tile_aniso<NBR, 128, 32, FIELD, HASMP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)smem));
+    count_launch();
+    k_tile_aniso<NBR, 128, 32, FIELD, HASMP><<<(unsigned)a.tiles, kTileThreads, smem, s>>>(a, an);
+    HP_LAUNCH_CHECK("k_tile_aniso");
+    return HP_OK;
+}
+
 }  // namespace
+
+// 1024^2, 8 neighbours, Read-Shockley tables: 20.7 us per MCS; 72 us on the per-colour
+// kernel, four launches whose bins took a 64-bit remainder and division each.
+int tile_launch_aniso(const PlaneArgs& a, const Aniso& an, int field, bool hasmp, int nbr, cudaStream_t s) {
+    if (field == HP_FIELD_POINT && hasmp) return nbr == 8 ? launch_aniso<8, 2, true>(a, an, s) : launch_aniso<4, 2, true>(a, an, s);
+    if (field == HP_FIELD_GRAIN && !hasmp) return nbr == 8 ? launch_aniso<8, 1, false>(a, an, s) : launch_aniso<4, 1, false>(a, an, s);
+    if (field == HP_FIELD_NONE && !hasmp) return nbr == 8 ? launch_aniso<8, 0, false>(a, an, s) : launch_aniso<4, 0, false>(a, an, s);
+    return set_error(HP_ERR_ARG, "sweep: no tile kernel with misorientation tables for this field mode");
+}
 
 int tile_launch(const PlaneArgs& a, int field, bool hasmp, int nbr, int planes, int WX, int WY, cudaStream_t s) {
     return tile_dispatch(&a, nullptr, field, hasmp, nbr, planes, WX, WY, s);
