@@ -9,10 +9,18 @@
 //
 // Assignment: each site takes the seed at the smallest periodic minimum-image
 // squared distance, ties to the lowest index.  Seeds are bucketed into a grid
-// of cells (about two seeds per cell); a site scans rings of cells of growing
-// Chebyshev radius r around its own cell and stops once the best squared
-// distance is below (r * wmin + 1)^2, the least squared distance any seed
-// outside the scanned rings can have (wmin = narrowest cell width).
+// of cells (about two seeds per cell); any seed outside the cells within Chebyshev
+// radius r of a set of cells is at least r * wmin + 1 (wmin = narrowest cell width)
+// away from every site in them.
+//
+// A block takes a brick of sites (k_assign_bricks).  With D(s) the largest distance
+// of seed s to any site of the brick, no site of it is further than U = min D(s)
+// from its nearest seed, so only seeds whose least distance to the brick is at most
+// U can be anyone's; rings of cells are added until U is below the bound above.
+// Every warp narrows the brick's list down in the same way to its runs of 32
+// adjacent sites, and its lanes then compare a handful of seeds each.  What bounds
+// it: integer instructions; the scan of the 27 cells around every site that it
+// replaces (54 seeds, 64-bit distances) took about 6000 per site.
 #include <math.h>
 
 
@@ -109,17 +117,12 @@ __device__ __forceinline__ int wrapc(int a, int n) {
     return a < 0 ? a + n : a;
 }
 
-__global__ void __launch_bounds__(kT) k_assign(int32_t* q, int32_t* mp, int64_t N, Cells c, const int32_t* start,
-                                               const int4* list) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= N) return;
-    const int x = (int)(i % c.L[0]);
-    const int y = (int)((i / c.L[0]) % c.L[1]);
-    const int z = (int)(i / ((int64_t)c.L[0] * c.L[1]));
+// Nearest seed of one site by its own rings of cells: what a brick with too many
+// seeds nearby, and lattices too long for 32-bit distances, fall back to.
+__device__ __noinline__ int32_t assign_site(int x, int y, int z, const Cells& c, const int32_t* start, const int4* list) {
     const int cx = cell_of(x, c.L[0], c.nc[0]), cy = cell_of(y, c.L[1], c.nc[1]), cz = cell_of(z, c.L[2], c.nc[2]);
     int64_t best = INT64_MAX;
     int32_t arg = INT32_MAX;
-    const int rz_max = c.dim == 3 ? 1 : 0;
     for (int r = 0;; ++r) {
         const int rz = c.dim == 3 ? r : 0;
         for (int dz = -rz; dz <= rz; ++dz) {
@@ -144,13 +147,281 @@ __global__ void __launch_bounds__(kT) k_assign(int32_t* q, int32_t* mp, int64_t 
                 }
             }
         }
-        (void)rz_max;
         const int64_t bound = (int64_t)r * c.wmin + 1;
         const bool all = (2 * r + 1 >= c.nc[0]) && (2 * r + 1 >= c.nc[1]) && (c.dim == 2 || 2 * r + 1 >= c.nc[2]);
         if ((arg != INT32_MAX && best < bound * bound) || all) break;
     }
-    q[i] = arg;
+    return arg;
+}
+
+__global__ void __launch_bounds__(kT) k_assign(int32_t* q, int32_t* mp, int64_t N, Cells c, const int32_t* start,
+                                               const int4* list) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= N) return;
+    const int x = (int)(i % c.L[0]);
+    const int y = (int)((i / c.L[0]) % c.L[1]);
+    const int z = (int)(i / ((int64_t)c.L[0] * c.L[1]));
+    q[i] = assign_site(x, y, z, c, start, list);
     if (mp) mp[i] = (int32_t)i;
+}
+
+// Least and largest periodic distance of coordinate s to the interval [b, b + len] of
+// an axis of (even, or 1) length L > len.
+struct Reach {
+    int lo, hi;
+};
+__device__ __forceinline__ Reach reach(int s, int b, int len, int L) {
+    int u = s - b;
+    u += u < 0 ? L : 0;  // 0 <= u < L
+    const int v = u > len ? u - len : len - u;
+    int h = u + (L >> 1);
+    h -= h >= L ? L : 0;  // offset of the point opposite to s
+    Reach r;
+    r.lo = u <= len ? 0 : min(u - len, L - u);
+    r.hi = h <= len ? L >> 1 : max(min(u, L - u), min(v, L - v));
+    return r;
+}
+struct Box {
+    int b[3], len[3];
+};
+// squared least and largest distances of seed s to the box
+__device__ __forceinline__ Reach reach2(const int4 s, const Box& k, const Cells& c) {
+    const Reach x = reach(s.x, k.b[0], k.len[0], c.L[0]), y = reach(s.y, k.b[1], k.len[1], c.L[1]),
+                z = reach(s.z, k.b[2], k.len[2], c.L[2]);
+    return Reach{x.lo * x.lo + y.lo * y.lo + z.lo * z.lo, x.hi * x.hi + y.hi * y.hi + z.hi * z.hi};
+}
+
+// Bricks of 32 x 8 x 8 sites (2D: 64 x 32), one warp run 8 x 4 x 2 (8 x 8), two sites
+// to a lane: compact, for a short list, and 32 bytes of a row, for whole sectors.
+// kNear seeds per brick and kRun per run; beyond, a run tests the brick's list and a
+// brick its sites' own rings.  256^3, 16000 seeds, whole call: 3.1 ms with the rings
+// per site.
+constexpr int kNear = 1024, kRun = 64;
+
+template <int DIM>
+struct Brick {
+    static constexpr int X = DIM == 3 ? 32 : 64, Y = DIM == 3 ? 8 : 32, Z = DIM == 3 ? 8 : 1;
+    static constexpr int RX = 8, RY = DIM == 3 ? 4 : 8, RZ = DIM == 3 ? 2 : 1;  // lanes: 8 x 4, twice (in z; in y)
+    static constexpr int NX = X / RX, NY = Y / RY, RUNS = NX * NY * (Z / RZ);
+};
+
+// The runs of a brick.  NEAR: the brick's seeds are given by the image closest to it,
+// which is the closest to each of its sites (the brick and its reach span no more than
+// half of any axis); otherwise every distance is folded.
+template <int DIM, bool NEAR>
+__device__ __forceinline__ void brick_runs(const Box& k, const Cells& c, const int4* near_, int n, int4* run,
+                                           int32_t* __restrict__ q, int32_t* __restrict__ mp) {
+    using B = Brick<DIM>;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const unsigned lt = (1u << lane) - 1u;
+    for (int t = warp; t < B::RUNS; t += kT / 32) {
+        Box m;
+        m.b[0] = k.b[0] + (t % B::NX) * B::RX;
+        m.b[1] = k.b[1] + (t / B::NX % B::NY) * B::RY;
+        m.b[2] = k.b[2] + (t / (B::NX * B::NY)) * B::RZ;
+        if (m.b[0] >= c.L[0] || m.b[1] >= c.L[1] || m.b[2] >= c.L[2]) continue;
+        const int full[3] = {B::RX, B::RY, B::RZ};
+        int end[3];
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            m.len[d] = min(full[d], c.L[d] - m.b[d]) - 1;
+            end[d] = m.b[d] + m.len[d];
+        }
+        auto reach_of = [&](const int4 s) {
+            if (!NEAR) return reach2(s, m, c);
+            const int sd[3] = {s.x, s.y, s.z};
+            Reach r{0, 0};
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+                if (DIM == 2 && d == 2) continue;
+                const int u = m.b[d] - sd[d], v = sd[d] - end[d];  // past either end
+                const int lo = max(max(u, v), 0), hi = m.len[d] - min(u, v);
+                r.lo += lo * lo;
+                r.hi += hi * hi;
+            }
+            return r;
+        };
+        // the first 64 seeds stay in registers between the two looks at them
+        int lo0 = INT32_MAX, lo1 = INT32_MAX, best = INT32_MAX;
+        if (lane < n) {
+            const Reach r = reach_of(near_[lane]);
+            lo0 = r.lo;
+            best = r.hi;
+        }
+        if (lane + 32 < n) {
+            const Reach r = reach_of(near_[lane + 32]);
+            lo1 = r.lo;
+            best = min(best, r.hi);
+        }
+        for (int i = lane + 64; i < n; i += 32) best = min(best, reach_of(near_[i]).hi);
+        best = __reduce_min_sync(0xFFFFFFFFu, best);
+        int nr = 0;
+        for (int i0 = 0; i0 < n; i0 += 32) {
+            const int i = i0 + lane;
+            int lo = i0 == 0 ? lo0 : lo1;
+            if (i0 >= 64) lo = i < n ? reach_of(near_[i]).lo : INT32_MAX;
+            const bool keep = lo <= best && i < n;
+            const unsigned bal = __ballot_sync(0xFFFFFFFFu, keep);
+            const int at = nr + __popc(bal & lt);
+            if (keep && at < kRun) run[at] = near_[i];
+            nr += __popc(bal);
+        }
+        __syncwarp();
+        const int4* src = nr <= kRun ? run : near_;
+        const int ns = nr <= kRun ? nr : n;
+        // lane's sites (x, y, z) and one further along z (3D) or four along y (2D)
+        const int x = m.b[0] + (lane & 7), y = m.b[1] + (lane >> 3), z = m.b[2];
+        const int y1 = DIM == 3 ? y : y + 4, z1 = DIM == 3 ? z + 1 : z;
+        int d0 = INT32_MAX, d1 = INT32_MAX, g0 = INT32_MAX, g1 = INT32_MAX;
+        for (int i = 0; i < ns; ++i) {
+            const int4 s = src[i];
+            int dx = x - s.x, dy = y - s.y, dz = z - s.z, ey = y1 - s.y, ez = z1 - s.z;
+            if (!NEAR) {
+                dx = abs(dx); dy = abs(dy); dz = abs(dz); ey = abs(ey); ez = abs(ez);
+                dx = min(dx, c.L[0] - dx);
+                dy = min(dy, c.L[1] - dy);
+                dz = min(dz, c.L[2] - dz);
+                ey = min(ey, c.L[1] - ey);
+                ez = min(ez, c.L[2] - ez);
+            }
+            const int a = dx * dx + (DIM == 3 ? dy * dy : 0), u = a + (DIM == 3 ? dz * dz : dy * dy),
+                      v = a + (DIM == 3 ? ez * ez : ey * ey);
+            if (u < d0 || (u == d0 && s.w < g0)) { d0 = u; g0 = s.w; }
+            if (v < d1 || (v == d1 && s.w < g1)) { d1 = v; g1 = s.w; }
+        }
+        __syncwarp();
+        if (x < c.L[0] && y < c.L[1]) {
+            const int64_t i = x + (int64_t)c.L[0] * (y + (int64_t)c.L[1] * z);
+            q[i] = g0;
+            if (mp) mp[i] = (int32_t)i;
+        }
+        if (x < c.L[0] && y1 < c.L[1] && z1 < c.L[2]) {
+            const int64_t i = x + (int64_t)c.L[0] * (y1 + (int64_t)c.L[1] * z1);
+            q[i] = g1;
+            if (mp) mp[i] = (int32_t)i;
+        }
+    }
+}
+
+template <int DIM>
+__global__ void __launch_bounds__(kT) k_assign_bricks(int32_t* __restrict__ q, int32_t* __restrict__ mp,
+                                                      const __grid_constant__ Cells c,
+                                                      const int32_t* __restrict__ start, const int4* __restrict__ list,
+                                                      int nbx, int nby) {
+    using B = Brick<DIM>;
+    __shared__ int4 near_[kNear];
+    __shared__ int4 run[kT / 32][kRun];
+    __shared__ int s_best, s_n;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int bx = (int)(blockIdx.x % (unsigned)nbx), br = (int)(blockIdx.x / (unsigned)nbx);
+    Box k;
+    k.b[0] = bx * B::X;
+    k.b[1] = (br % nby) * B::Y;
+    k.b[2] = (br / nby) * B::Z;
+    const int ext[3] = {B::X, B::Y, B::Z};
+    int c0[3], nc[3];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        k.len[d] = min(ext[d], c.L[d] - k.b[d]) - 1;
+        c0[d] = cell_of(k.b[d], c.L[d], c.nc[d]);
+        nc[d] = cell_of(k.b[d] + k.len[d], c.L[d], c.nc[d]) - c0[d] + 1;
+    }
+    // seeds of the cells within radius r of the brick's, by rows of cells along x (one
+    // or, across the edge, two runs of the list): f(seed) for every one of them
+    auto scan = [&](int r, auto f) {
+        int n[3], f0[3];
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            const int rr = d == 2 && DIM == 2 ? 0 : r;
+            n[d] = min(nc[d] + 2 * rr, c.nc[d]);
+            f0[d] = n[d] == c.nc[d] ? 0 : c0[d] - rr;  // rr < nc: at most one period below 0
+            f0[d] += f0[d] < 0 ? c.nc[d] : 0;
+        }
+        const int first = min(n[0], c.nc[0] - f0[0]);  // cells before the edge
+        for (int row = warp; row < n[1] * n[2]; row += kT / 32) {
+            const int rz = DIM == 3 ? (int)((unsigned)row / (unsigned)n[1]) : 0;
+            int cy = f0[1] + row - rz * n[1], cz = f0[2] + rz;
+            cy -= cy >= c.nc[1] ? c.nc[1] : 0;
+            cz -= cz >= c.nc[2] ? c.nc[2] : 0;
+            const int32_t* st = start + (int64_t)c.nc[0] * (cy + (int64_t)c.nc[1] * cz);
+            int s0 = st[f0[0]], s1 = st[f0[0] + first];
+            for (int i = s0 + lane; i < s1; i += 32) f(list[i]);
+            if (first < n[0]) {
+                s0 = st[0];
+                s1 = st[n[0] - first];
+                for (int i = s0 + lane; i < s1; i += 32) f(list[i]);
+            }
+        }
+        return n[0] == c.nc[0] && n[1] == c.nc[1] && n[2] == c.nc[2];
+    };
+    if (tid == 0) {
+        s_best = INT32_MAX;
+        s_n = 0;
+    }
+    __syncthreads();
+    int r = 1, far2;
+    for (;; ++r) {
+        int best = INT32_MAX;
+        const bool all = scan(r, [&](const int4 s) { best = min(best, reach2(s, k, c).hi); });
+        best = __reduce_min_sync(0xFFFFFFFFu, best);
+        if (lane == 0) atomicMin(&s_best, best);
+        __syncthreads();
+        far2 = s_best;
+        const int64_t bound = (int64_t)r * c.wmin + 1;
+        if (all || (int64_t)far2 < bound * bound) break;
+        __syncthreads();
+    }
+    // no distance looked at below exceeds U + the brick's length, U = sqrt(far2)
+    const int U = (int)sqrtf((float)far2) + 2;
+    bool near = true;
+#pragma unroll
+    for (int d = 0; d < DIM; ++d) near &= U + k.len[d] <= c.L[d] / 2;
+    scan(r, [&](int4 s) {
+        if (reach2(s, k, c).lo > far2) return;
+        if (near) {  // the image closest to the brick
+            int* sd[3] = {&s.x, &s.y, &s.z};
+#pragma unroll
+            for (int d = 0; d < DIM; ++d) {
+                int u = *sd[d] - k.b[d];
+                u += u < 0 ? c.L[d] : 0;
+                *sd[d] = k.b[d] + (u > k.len[d] && u - k.len[d] > c.L[d] - u ? u - c.L[d] : u);
+            }
+        }
+        const int i = atomicAdd(&s_n, 1);
+        if (i < kNear) near_[i] = s;
+    });
+    __syncthreads();
+    const int n = s_n;
+    if (n <= kNear) {
+        if (near) brick_runs<DIM, true>(k, c, near_, n, run[warp], q, mp);
+        else brick_runs<DIM, false>(k, c, near_, n, run[warp], q, mp);
+        return;
+    }
+    for (int t = tid; t < B::X * B::Y * B::Z; t += kT) {
+        const int x = k.b[0] + t % B::X, y = k.b[1] + t / B::X % B::Y, z = k.b[2] + t / (B::X * B::Y);
+        if (x >= c.L[0] || y >= c.L[1] || z >= c.L[2]) continue;
+        const int64_t i = x + (int64_t)c.L[0] * (y + (int64_t)c.L[1] * z);
+        q[i] = assign_site(x, y, z, c, start, list);
+        if (mp) mp[i] = (int32_t)i;
+    }
+}
+
+// Bricks where squared distances stay below 2^31 (axes up to 32768), single sites
+// otherwise.
+void launch_assign(int32_t* q, int32_t* mp, int64_t N, const Cells& c, const int32_t* start, const int4* list,
+                   cudaStream_t s) {
+    ::hp::count_launch();
+    if (c.L[0] > 32768 || c.L[1] > 32768 || c.L[2] > 32768) {
+        k_assign<<<(unsigned)((N + kT - 1) / kT), kT, 0, s>>>(q, mp, N, c, start, list);
+    } else if (c.dim == 3) {
+        using B = Brick<3>;
+        const int nx = (c.L[0] + B::X - 1) / B::X, ny = (c.L[1] + B::Y - 1) / B::Y, nz = (c.L[2] + B::Z - 1) / B::Z;
+        k_assign_bricks<3><<<(unsigned)nx * ny * nz, kT, 0, s>>>(q, mp, c, start, list, nx, ny);
+    } else {
+        using B = Brick<2>;
+        const int nx = (c.L[0] + B::X - 1) / B::X, ny = (c.L[1] + B::Y - 1) / B::Y;
+        k_assign_bricks<2><<<(unsigned)nx * ny, kT, 0, s>>>(q, mp, c, start, list, nx, ny);
+    }
 }
 
 __global__ void k_orient(int32_t G, uint64_t seed, int32_t kind, float* out) {
@@ -213,23 +484,20 @@ int voronoi_run(hp_handle* h, int32_t orient_kind, float* orient, int64_t* seed_
         const int w = c.L[d] / n;  // narrowest cell width along d
         c.wmin = w < c.wmin ? w : c.wmin;
     }
-    int64_t* pos = seed_pos;
-    int64_t* pos_own = nullptr;
-    int4 *xyz = nullptr, *list = nullptr;
-    int32_t *cnt = nullptr, *start = nullptr, *cursor = nullptr, *n_left = nullptr;
-    auto cleanup = [&]() {
-        cudaFreeAsync(pos_own, s); cudaFreeAsync(xyz, s); cudaFreeAsync(list, s);
-        cudaFreeAsync(cnt, s); cudaFreeAsync(start, s); cudaFreeAsync(cursor, s); cudaFreeAsync(n_left, s);
-    };
-    cudaError_t e = cudaSuccess;
-    if (!pos) e = cudaMallocAsync((void**)&pos_own, sizeof(int64_t) * G, s), pos = pos_own;
-    if (e == cudaSuccess) e = cudaMallocAsync((void**)&xyz, sizeof(int4) * G, s);
-    if (e == cudaSuccess) e = cudaMallocAsync((void**)&list, sizeof(int4) * G, s);
-    if (e == cudaSuccess) e = cudaMallocAsync((void**)&cnt, sizeof(int32_t) * ncell, s);
-    if (e == cudaSuccess) e = cudaMallocAsync((void**)&start, sizeof(int32_t) * (ncell + 1), s);
-    if (e == cudaSuccess) e = cudaMallocAsync((void**)&cursor, sizeof(int32_t) * ncell, s);
-    if (e == cudaSuccess) e = cudaMallocAsync((void**)&n_left, sizeof(int32_t), s);
-    if (e != cudaSuccess) { cleanup(); return set_error(HP_ERR_OOM, "hp_init_voronoi: scratch allocation failed"); }
+    // one allocation, carved (seven of them cost more than the kernels of a small call)
+    size_t bytes = 0;
+    auto take = [&](size_t n) { const size_t at = bytes; bytes += (n + 255) & ~(size_t)255; return at; };
+    const size_t o_xyz = take(sizeof(int4) * G), o_list = take(sizeof(int4) * G), o_cnt = take(sizeof(int32_t) * ncell),
+                 o_start = take(sizeof(int32_t) * (ncell + 1)), o_cursor = take(sizeof(int32_t) * ncell),
+                 o_left = take(sizeof(int32_t)), o_pos = take(seed_pos ? 0 : sizeof(int64_t) * G);
+    unsigned char* buf = nullptr;
+    cudaError_t e = cudaMallocAsync((void**)&buf, bytes, s);
+    auto cleanup = [&]() { cudaFreeAsync(buf, s); };
+    if (e != cudaSuccess) return set_error(HP_ERR_OOM, "hp_init_voronoi: scratch allocation failed");
+    int64_t* pos = seed_pos ? seed_pos : (int64_t*)(buf + o_pos);
+    int4 *xyz = (int4*)(buf + o_xyz), *list = (int4*)(buf + o_list);
+    int32_t *cnt = (int32_t*)(buf + o_cnt), *start = (int32_t*)(buf + o_start), *cursor = (int32_t*)(buf + o_cursor),
+            *n_left = (int32_t*)(buf + o_left);
 
     int rc = HP_OK;
     do {
@@ -257,9 +525,7 @@ int voronoi_run(hp_handle* h, int32_t orient_kind, float* orient, int64_t* seed_
         k_scan<<<1, 1024, 0, s>>>(cnt, start, (int32_t)ncell);
         ::hp::count_launch();
         k_cell_scatter<<<gb, kT, 0, s>>>(xyz, G, start, cursor, list);
-        const int64_t nb = (N + kT - 1) / kT;
-        ::hp::count_launch();
-        k_assign<<<(unsigned)nb, kT, 0, s>>>(h->q, h->mp, N, c, start, list);
+        launch_assign(h->q, h->mp, N, c, start, list, s);
         if ((e = cudaGetLastError())) break;
         if (orient) {
             ::hp::count_launch();
@@ -388,9 +654,7 @@ extern "C" int hp_init_voronoi_static(hp_handle* h, int32_t orient_kind, float* 
     k_scan<<<1, 1024, 0, s>>>(cnt, start, (int32_t)ncell);
     ::hp::count_launch();
     k_cell_scatter<<<gb, kT, 0, s>>>(xyz, G, start, cursor, list);
-    const int64_t nb = (N + kT - 1) / kT;
-    ::hp::count_launch();
-    k_assign<<<(unsigned)nb, kT, 0, s>>>(h->q, h->mp, N, c, start, list);
+    launch_assign(h->q, h->mp, N, c, start, list, s);
     if (orient) {
         ::hp::count_launch();
         k_orient<<<gb, kT, 0, s>>>(G, h->desc.seed, orient_kind, orient);
