@@ -9,7 +9,8 @@
 // the planes z-1 and z+1 are read-only neighbours (old for even planes, new for
 // odd planes), exactly as in the plane kernel, and each MCS is two launches.
 //
-// Per phase:
+// Per phase (a warp at a time where a row is one warp wide, 8 neighbours; the block
+// together otherwise):
 //   A. the phase's (row, quad) items go out in chunks of 64 per warp trip, two
 //      per lane; a lane keeps one aligned quad of four columns.  One 128-bit
 //      shared load per neighbour row, with the edge columns taken from the
@@ -49,7 +50,10 @@ struct TileCfg {
     static constexpr int PAD = 8;                  // ints of padding before and after each array
     static constexpr int AS = WX * WY + 2 * PAD;   // array stride in ints
     static constexpr int QPR = WX / 4;             // quads per row (a lane keeps its quad)
-    static constexpr int QCAP = NBR == 4 ? (WX / 2) * WY : (WX / 2) * ((WY + 1) / 2);
+    // 8 neighbours, rows of one warp's width: row pairs per warp
+    static constexpr bool ROWS = NBR == 8 && WX == 128 && WY % 32 == 0;
+    static constexpr int PER = WY / 16;
+    static constexpr int QCAP = ROWS ? PER * 64 * 8 / 2 : NBR == 4 ? (WX / 2) * WY : (WX / 2) * ((WY + 1) / 2);
     static_assert(WX % 4 == 0 && (AS * 4) % 16 == 0 && 32 % QPR == 0 && TY % 2 == 0, "tile shape");
     __host__ __device__ static constexpr int ylo(int p) { return NBR == 4 ? p + 1 : 1 + (p >> 1); }
     static size_t smem() { return 128 + sizeof(int32_t) * ((size_t)ARR * AS + QCAP + 8) + sizeof(uint2) * 64 * (kTileThreads / 32); }
@@ -238,62 +242,108 @@ __device__ __forceinline__ void tile_body(const PlaneArgs& a, const int tile, co
     const int warp = (int)(threadIdx.x >> 5);
     const int c0 = 4 * (lane % QPR);
     const uint32_t cz = Z ? 4u * (uint32_t)a.zpar : 0u;
+    // one quad of row r: sites ca = c0 + px and cb = ca + 2; bits 0/1 of
+    // the result say which of them need the Metropolis stage
+    auto item = [&](const int p, const int r, int& ca, int& cb) -> uint32_t {
+        const int lo = p + 1, hi = WX - p - 1, hiy = WY - Cfg::ylo(p);
+        const int px = NBR == 4 ? ((r + p) & 1) : (p & 1);
+        const int ca_ = c0 + px, cb_ = ca_ + 2;
+        const bool rowok = r < hiy;
+        const bool va = rowok && ca_ >= lo && ca_ < hi;
+        const bool vb = rowok && cb_ >= lo && cb_ < hi;
+        // every lane loads (lanes past the last row read row hiy - 1 and
+        // discard it) so that the edge columns can come from the
+        // neighbouring lanes: the left lane's last column and the right
+        // lane's first.  A lane at the end of a warp row only ever holds a
+        // site outside [lo, hi) on that side.
+        const int rowq = (rowok ? r : hiy - 1) * WX + c0;
+        const int32_t* own = t.S + rowq;
+        const int4 cv = *reinterpret_cast<const int4*>(own);
+        const int32_t q0 = px ? cv.y : cv.x, q1 = px ? cv.w : cv.z;
+        uint32_t acc0 = 0, acc1 = 0;
+        // the three columns around each site in one row (values v)
+        auto cols = [&](const int4 v, bool centre) {
+            const int32_t el = __shfl_up_sync(0xFFFFFFFFu, v.w, 1);
+            const int32_t er = __shfl_down_sync(0xFFFFFFFFu, v.x, 1);
+            const int32_t l0 = px ? v.x : el, m0 = px ? v.y : v.x, r0_ = px ? v.z : v.y;
+            const int32_t l1 = px ? v.z : v.y, m1 = px ? v.w : v.z, r1 = px ? er : v.w;
+            acc0 |= (l0 ^ q0) | (r0_ ^ q0);
+            acc1 |= (l1 ^ q1) | (r1 ^ q1);
+            if (!centre) { acc0 |= m0 ^ q0; acc1 |= m1 ^ q1; }
+        };
+        auto ld = [&](const int32_t* P) { return *reinterpret_cast<const int4*>(P); };
+        if (NBR == 4) {
+            cols(cv, true);
+            const int4 u = ld(own - WX), d = ld(own + WX);
+            acc0 |= ((px ? u.y : u.x) ^ q0) | ((px ? d.y : d.x) ^ q0);
+            acc1 |= ((px ? u.w : u.z) ^ q1) | ((px ? d.w : d.z) ^ q1);
+        } else {
+            cols(ld(own - WX), false);
+            cols(cv, true);
+            cols(ld(own + WX), false);
+            if (Z) {
+#pragma unroll
+                for (int dy = -1; dy <= 1; ++dy) {
+                    cols(ld(t.SLO + rowq + dy * WX), false);
+                    cols(ld(t.SHI + rowq + dy * WX), false);
+                }
+            }
+        }
+        ca = ca_;
+        cb = cb_;
+        return (va && acc0 != 0u ? 1u : 0u) | (vb && acc1 != 0u ? 2u : 0u);
+    };
+    if constexpr (Cfg::ROWS) {
+        // Phases 0 and 1 (even rows) meet the odd rows only as unchanged neighbours, and
+        // phases 2 and 3 the even rows, so a warp that owns whole rows (pairs 2j, 2j + 1
+        // with j = warp, warp + 8, ..) queues, draws and tests on its own, and the block
+        // meets once, between phases 1 and 2 (4096^2: 66.4 -> 63.8 us per MCS against
+        // the block-wide queue below; what is left at barriers is the wait for the
+        // window, a quarter of all stall samples).
+        uint16_t* wl = reinterpret_cast<uint16_t*>(queue) + Cfg::PER * 64 * warp;
+        uint2* wq = wqueue + 64 * warp;
+#pragma unroll
+        for (int p = 0; p < 4; ++p) {
+            int n = 0;
+#pragma unroll
+            for (int m = 0; m < Cfg::PER; m += 2) {
+                const int r1 = 2 * (warp + 8 * m) + (p >> 1), r2 = r1 + 16, loy = 1 + (p >> 1);
+                int ca1, cb1, ca2, cb2;
+                uint32_t f1 = item(p, max(r1, loy), ca1, cb1), f2 = item(p, r2, ca2, cb2);
+                if (r1 < loy) f1 = 0;
+                const unsigned m0 = __ballot_sync(0xFFFFFFFFu, f1 & 1u), m1 = __ballot_sync(0xFFFFFFFFu, f1 & 2u);
+                const unsigned m2 = __ballot_sync(0xFFFFFFFFu, f2 & 1u), m3 = __ballot_sync(0xFFFFFFFFu, f2 & 2u);
+                const int n0 = n + __popc(m0), n1 = n0 + __popc(m1), n2 = n1 + __popc(m2);
+                if (f1 & 1u) wl[n + __popc(m0 & lt)] = (uint16_t)((r1 << 8) | ca1);
+                if (f1 & 2u) wl[n0 + __popc(m1 & lt)] = (uint16_t)((r1 << 8) | cb1);
+                if (f2 & 1u) wl[n1 + __popc(m2 & lt)] = (uint16_t)((r2 << 8) | ca2);
+                if (f2 & 2u) wl[n2 + __popc(m3 & lt)] = (uint16_t)((r2 << 8) | cb2);
+                n = n2 + __popc(m3);
+            }
+            __syncwarp();
+            for (int k0 = 0; k0 < n; k0 += 64) {
+                const int k1 = k0 + lane, k2 = k1 + 32;
+                uint2 w1 = make_uint2(0u, 0u), w2 = make_uint2(0u, 0u);
+                const bool a1 = k1 < n && t.draw_site(wl[k1], (uint32_t)p, w1);
+                const bool a2 = k2 < n && t.draw_site(wl[k2], (uint32_t)p, w2);
+                const unsigned m1 = __ballot_sync(0xFFFFFFFFu, a1), m2 = __ballot_sync(0xFFFFFFFFu, a2);
+                if (a1) wq[__popc(m1 & lt)] = w1;
+                if (a2) wq[__popc(m1) + __popc(m2 & lt)] = w2;
+                __syncwarp();
+                const int na = __popc(m1) + __popc(m2);
+                for (int j = lane; j < na; j += 32) t.test(wq[j]);
+                __syncwarp();
+            }
+            if (p == 1) __syncthreads(); else __syncwarp();
+        }
+        __syncthreads();
+    } else {
 #pragma unroll
     for (int p = 0; p < NP; ++p) {
-        const int lo = p + 1, hi = WX - p - 1, loy = Cfg::ylo(p), hiy = WY - loy;
+        const int loy = Cfg::ylo(p), hiy = WY - loy;
         // ---- A: interior test, queue the rest ---------------------------------
         constexpr int RSTEP = NBR == 4 ? 1 : 2;
         const int rstart = NBR == 4 ? loy : loy + ((loy ^ (p >> 1)) & 1);
-        // one quad of row r: sites ca = c0 + px and cb = ca + 2; bits 0/1 of
-        // the result say which of them need the Metropolis stage
-        auto item = [&](const int r, int& ca, int& cb) -> uint32_t {
-            const int px = NBR == 4 ? ((r + p) & 1) : (p & 1);
-            const int ca_ = c0 + px, cb_ = ca_ + 2;
-            const bool rowok = r < hiy;
-            const bool va = rowok && ca_ >= lo && ca_ < hi;
-            const bool vb = rowok && cb_ >= lo && cb_ < hi;
-            // every lane loads (lanes past the last row read row hiy - 1 and
-            // discard it) so that the edge columns can come from the
-            // neighbouring lanes: the left lane's last column and the right
-            // lane's first.  A lane at the end of a warp row only ever holds a
-            // site outside [lo, hi) on that side.
-            const int rowq = (rowok ? r : hiy - 1) * WX + c0;
-            const int32_t* own = t.S + rowq;
-            const int4 cv = *reinterpret_cast<const int4*>(own);
-            const int32_t q0 = px ? cv.y : cv.x, q1 = px ? cv.w : cv.z;
-            uint32_t acc0 = 0, acc1 = 0;
-            // the three columns around each site in one row (values v)
-            auto cols = [&](const int4 v, bool centre) {
-                const int32_t el = __shfl_up_sync(0xFFFFFFFFu, v.w, 1);
-                const int32_t er = __shfl_down_sync(0xFFFFFFFFu, v.x, 1);
-                const int32_t l0 = px ? v.x : el, m0 = px ? v.y : v.x, r0_ = px ? v.z : v.y;
-                const int32_t l1 = px ? v.z : v.y, m1 = px ? v.w : v.z, r1 = px ? er : v.w;
-                acc0 |= (l0 ^ q0) | (r0_ ^ q0);
-                acc1 |= (l1 ^ q1) | (r1 ^ q1);
-                if (!centre) { acc0 |= m0 ^ q0; acc1 |= m1 ^ q1; }
-            };
-            auto ld = [&](const int32_t* P) { return *reinterpret_cast<const int4*>(P); };
-            if (NBR == 4) {
-                cols(cv, true);
-                const int4 u = ld(own - WX), d = ld(own + WX);
-                acc0 |= ((px ? u.y : u.x) ^ q0) | ((px ? d.y : d.x) ^ q0);
-                acc1 |= ((px ? u.w : u.z) ^ q1) | ((px ? d.w : d.z) ^ q1);
-            } else {
-                cols(ld(own - WX), false);
-                cols(cv, true);
-                cols(ld(own + WX), false);
-                if (Z) {
-#pragma unroll
-                    for (int dy = -1; dy <= 1; ++dy) {
-                        cols(ld(t.SLO + rowq + dy * WX), false);
-                        cols(ld(t.SHI + rowq + dy * WX), false);
-                    }
-                }
-            }
-            ca = ca_;
-            cb = cb_;
-            return (va && acc0 != 0u ? 1u : 0u) | (vb && acc1 != 0u ? 2u : 0u);
-        };
         // the phase's (row, quad) items in chunks of 64, one chunk per warp
         // trip, two items per lane whose loads and shuffles overlap; a lane
         // keeps its quad, so both items and all chunks share its columns
@@ -301,8 +351,8 @@ __device__ __forceinline__ void tile_body(const PlaneArgs& a, const int tile, co
         for (int ch = warp; 64 * ch < nitems; ch += kTileThreads / 32) {
             const int r1 = rstart + RSTEP * ((64 * ch + lane) / QPR), r2 = r1 + RSTEP * (32 / QPR);
             int ca1, cb1, ca2, cb2;
-            const uint32_t f1 = item(r1, ca1, cb1);
-            const uint32_t f2 = item(r2, ca2, cb2);
+            const uint32_t f1 = item(p, r1, ca1, cb1);
+            const uint32_t f2 = item(p, r2, ca2, cb2);
             const unsigned m0 = __ballot_sync(0xFFFFFFFFu, f1 & 1u), m1 = __ballot_sync(0xFFFFFFFFu, f1 & 2u);
             const unsigned m2 = __ballot_sync(0xFFFFFFFFu, f2 & 1u), m3 = __ballot_sync(0xFFFFFFFFu, f2 & 2u);
             if (m0 | m1 | m2 | m3) {
@@ -339,6 +389,7 @@ __device__ __forceinline__ void tile_body(const PlaneArgs& a, const int tile, co
             __syncwarp();
         }
         __syncthreads();
+    }
     }
     (void)M;
 
