@@ -103,8 +103,6 @@ extern "C" int hp_destroy(hp_handle* h) {
     cudaFree(h->an_J);
     cudaFree(h->an_mob);
     cudaFree(h->m_counts);
-    cudaFree(h->m_bins);
-    cudaFree(h->m_small);
     delete h;
     return HP_OK;
 }

@@ -164,9 +164,7 @@ struct hp_handle {
     uint32_t* an_mob = nullptr;
     int32_t an_period = 0, an_bin = 0, an_nbins = 0;
     // owned scratch of hp_measure (allocated on its first call)
-    unsigned long long* m_counts = nullptr;  // int64[G]
-    int32_t* m_bins = nullptr;               // int32[2G]
-    unsigned long long* m_small = nullptr;   // hist[90] | field sum | alive | bad ids
+    unsigned long long* m_counts = nullptr;  // counts[G] | hist[90] | field sum | alive | bad ids
 };
 
 namespace hp {

@@ -79,28 +79,54 @@ __global__ void k_grain_field(FieldArgs a) {
     if (a.mmax) a.mmax[g] = (float)mm;
 }
 
-// Per-grain counts: each thread scans a run of consecutive sites and adds the
-// length of each run of equal ids with one atomic.
-constexpr int kSeg = 32;
+// Per-grain counts, one atomic per run of equal ids along the array.  A warp reads 128
+// consecutive sites at a time, 16 bytes a lane where the array lies on a 16-byte
+// boundary (a thread that scans 32 sites by itself makes every load of a warp touch
+// 32 lines), finds the run starts with four ballots, and a start's run ends at the
+// next one.
+constexpr int kSeg = 2048;  // sites per warp
 
 __global__ void __launch_bounds__(kT) k_counts(const int32_t* __restrict__ q, int64_t N, int32_t G,
                                                unsigned long long* counts, int32_t* bad) {
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t b = t * kSeg;
-    if (b >= N) return;
-    const int64_t e = b + kSeg < N ? b + kSeg : N;
-    int32_t cur = q[b];
-    unsigned long long run = 0;
-    for (int64_t i = b; i < e; ++i) {
-        const int32_t v = q[i];
-        if (v != cur) {
-            if ((uint32_t)cur < (uint32_t)G) atomicAdd(counts + cur, run); else atomicAdd(bad, 1);
-            cur = v;
-            run = 0;
+    const int lane = threadIdx.x & 31;
+    const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const bool vec = ((uintptr_t)q & 15u) == 0;
+    const int64_t end = min((w + 1) * kSeg, N);
+    for (int64_t b = w * kSeg; b < end; b += 128) {
+        const int64_t at = b + 4 * lane;
+        const int n = (int)min((int64_t)128, end - b);  // sites of this step
+        int32_t v[4];
+        if (vec && at + 4 <= end) {
+            const int4 x = __ldg(reinterpret_cast<const int4*>(q + at));
+            v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
+        } else {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) v[i] = at + i < end ? __ldg(q + at + i) : 0;
         }
-        ++run;
+        // first[i]: lanes whose site i starts a run
+        const int32_t left = __shfl_up_sync(0xFFFFFFFFu, v[3], 1);
+        unsigned first[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int s = 4 * lane + i;
+            first[i] = __ballot_sync(0xFFFFFFFFu, s < n && (s == 0 || v[i] != (i ? v[i - 1] : left)));
+        }
+        const unsigned any = first[0] | first[1] | first[2] | first[3];
+        const unsigned later = lane == 31 ? 0u : any & (0xFFFFFFFEu << lane);  // lanes behind this one with a start
+        int stop = n;
+        if (later) {
+            const int l = __ffs(later) - 1;
+            stop = 4 * l + (first[0] >> l & 1u ? 0 : first[1] >> l & 1u ? 1 : first[2] >> l & 1u ? 2 : 3);
+        }
+#pragma unroll
+        for (int i = 3; i >= 0; --i) {
+            if (!(first[i] >> lane & 1u)) continue;
+            const int s = 4 * lane + i;
+            if ((uint32_t)v[i] < (uint32_t)G) atomicAdd(counts + v[i], (unsigned long long)(stop - s));
+            else atomicAdd(bad, 1);
+            stop = s;
+        }
     }
-    if ((uint32_t)cur < (uint32_t)G) atomicAdd(counts + cur, run); else atomicAdd(bad, 1);
 }
 
 __global__ void k_alive(const unsigned long long* counts, int32_t G, int32_t* alive) {
@@ -110,16 +136,16 @@ __global__ void k_alive(const unsigned long long* counts, int32_t G, int32_t* al
     if (threadIdx.x == 0 && s) atomicAdd(alive, s);
 }
 
-__global__ void k_bins(int32_t G, int32_t kind, const float* orient, int32_t* bins) {
-    const int32_t g = blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= G) return;
+// texture bins of grain g; b1 is -1 but for HP_ORIENT_SO3
+__device__ __forceinline__ void orient_bins(int32_t kind, const float* orient, int32_t g, int32_t* b0, int32_t* b1) {
     const double pi = 3.14159265358979323846;
+    *b1 = -1;
     if (kind == HP_ORIENT_ANGLE || kind == HP_ORIENT_ZROT) {
         const double t = kind == HP_ORIENT_ANGLE ? (double)orient[g]
                                                  : 2.0 * atan2((double)orient[4 * g + 3], (double)orient[4 * g]);
         const double deg = t * (180.0 / pi);
-        int b = (int)floor(deg);
-        bins[g] = b < 0 ? 0 : (b > 89 ? 89 : b);
+        const int b = (int)floor(deg);
+        *b0 = b < 0 ? 0 : (b > 89 ? 89 : b);
         return;
     }
     double d[3];
@@ -128,8 +154,8 @@ __global__ void k_bins(int32_t G, int32_t kind, const float* orient, int32_t* bi
     const double a0 = fabs(d[0] / nn), a1 = fabs(d[1] / nn), a2 = fabs(d[2] / nn);
     const double ad[3] = {a0, a1, a2};
     const double v = max_schmid(ad) / 0.5 * 20.0;
-    int b = (int)floor(v);
-    bins[2 * g] = b < 0 ? 0 : (b > 19 ? 19 : b);
+    const int b = (int)floor(v);
+    *b0 = b < 0 ? 0 : (b > 19 ? 19 : b);
     const double c15 = cos(15.0 * pi / 180.0);
     const double c100 = fmax(a0, fmax(a1, a2));
     const double c110 = fmax(a0 + a1, fmax(a1 + a2, a0 + a2)) / sqrt(2.0);
@@ -138,7 +164,20 @@ __global__ void k_bins(int32_t G, int32_t kind, const float* orient, int32_t* bi
     if (c100 > c15) fam = 1;
     else if (c110 > c15) fam = 2;
     else if (c111 > c15) fam = 3;
-    bins[2 * g + 1] = 20 + fam;
+    *b1 = 20 + fam;
+}
+
+__global__ void k_bins(int32_t G, int32_t kind, const float* orient, int32_t* bins) {
+    const int32_t g = blockIdx.x * blockDim.x + threadIdx.x;
+    if (g >= G) return;
+    int32_t b0, b1;
+    orient_bins(kind, orient, g, &b0, &b1);
+    if (b1 < 0) {
+        bins[g] = b0;
+    } else {
+        bins[2 * g] = b0;
+        bins[2 * g + 1] = b1;
+    }
 }
 
 __global__ void k_hist(int32_t G, int32_t kind, const int32_t* bins, const unsigned long long* counts,
@@ -185,11 +224,29 @@ __device__ __forceinline__ void block_add(long long v, unsigned long long* sum) 
     }
 }
 
-// Volume-weighted field sum, per-grain table: sum_g counts[g] table[g].
-__global__ void __launch_bounds__(kT) k_field_sum_grain(const unsigned long long* counts, const int32_t* table,
-                                                        int32_t G, unsigned long long* sum) {
+// What hp_measure derives from the counts, in one pass over the grains: grains alive,
+// the texture histogram (bins as k_bins gives them) and the volume-weighted field of a
+// per-grain table, each gathered per block before it goes to global memory.
+__global__ void __launch_bounds__(kT) k_grain_stats(const unsigned long long* __restrict__ counts, int32_t G, int32_t kind,
+                                                    const float* __restrict__ orient, const int32_t* __restrict__ table,
+                                                    unsigned long long* hist, unsigned long long* field, int32_t* alive) {
+    __shared__ unsigned long long h[90];
+    for (int i = threadIdx.x; i < 90; i += kT) h[i] = 0;
+    __syncthreads();
     const int32_t g = blockIdx.x * blockDim.x + threadIdx.x;
-    block_add(g < G ? (long long)counts[g] * (long long)table[g] : 0ll, sum);
+    const unsigned long long n = g < G ? counts[g] : 0ull;
+    if (n && orient) {
+        int32_t b0, b1;
+        orient_bins(kind, orient, g, &b0, &b1);
+        atomicAdd(h + b0, n);
+        if (b1 >= 0) atomicAdd(h + b1, n);
+    }
+    const int live = __syncthreads_count(n > 0);
+    if (threadIdx.x == 0 && live) atomicAdd(alive, live);
+    if (orient)
+        for (int i = threadIdx.x; i < 90; i += kT)
+            if (h[i]) atomicAdd(hist + i, h[i]);
+    if (table) block_add(n ? (long long)n * (long long)table[g] : 0ll, field);
 }
 
 // Per-point table: sum_i table[mp_i] (index clamped into the table).
@@ -252,6 +309,8 @@ extern "C" int hp_grain_field(int32_t G, const float* quat, double C11, double C
     return HP_OK;
 }
 
+static unsigned counts_grid(int64_t N) { return (unsigned)(((N + kSeg - 1) / kSeg * 32 + kT - 1) / kT); }
+
 extern "C" int hp_grain_counts(hp_handle* h, int64_t* counts, int32_t* alive, void* stream) {
     hp::Range r_("hp_grain_counts");
     if (!h || !counts) return set_error(HP_ERR_ARG, "hp_grain_counts: bad arguments");
@@ -262,10 +321,8 @@ extern "C" int hp_grain_counts(hp_handle* h, int64_t* counts, int32_t* alive, vo
     int32_t* bad = nullptr;
     HP_CUDA(cudaMallocAsync((void**)&bad, sizeof(int32_t), s));
     cudaMemsetAsync(bad, 0, sizeof(int32_t), s);
-    const int64_t threads = (h->lat.N + kSeg - 1) / kSeg;
     ::hp::count_launch();
-    k_counts<<<(unsigned)((threads + kT - 1) / kT), kT, 0, s>>>(h->q, h->lat.N, G,
-                                                                reinterpret_cast<unsigned long long*>(counts), bad);
+    k_counts<<<counts_grid(h->lat.N), kT, 0, s>>>(h->q, h->lat.N, G, reinterpret_cast<unsigned long long*>(counts), bad);
     if (alive) {
         cudaMemsetAsync(alive, 0, sizeof(int32_t), s);
         ::hp::count_launch();
@@ -315,30 +372,20 @@ extern "C" int hp_measure(hp_handle* h, int32_t orient_kind, const float* orient
         return set_error(HP_ERR_STATE, "hp_measure: no field table set");
     const int32_t G = h->desc.n_grains;
     cudaStream_t s = as_stream(stream);
-    if (!h->m_counts) HP_CUDA(cudaMalloc((void**)&h->m_counts, sizeof(unsigned long long) * (size_t)G));
-    if (!h->m_bins) HP_CUDA(cudaMalloc((void**)&h->m_bins, sizeof(int32_t) * 2 * (size_t)G));
-    if (!h->m_small) HP_CUDA(cudaMalloc((void**)&h->m_small, sizeof(unsigned long long) * kSlots));
-    unsigned long long* sm = h->m_small;
-    HP_CUDA(cudaMemsetAsync(h->m_counts, 0, sizeof(unsigned long long) * (size_t)G, s));
-    HP_CUDA(cudaMemsetAsync(sm, 0, sizeof(unsigned long long) * kSlots, s));
+    // counts, then the small slots: one buffer, cleared at once
+    if (!h->m_counts) HP_CUDA(cudaMalloc((void**)&h->m_counts, sizeof(unsigned long long) * ((size_t)G + kSlots)));
+    unsigned long long* sm = h->m_counts + G;
+    HP_CUDA(cudaMemsetAsync(h->m_counts, 0, sizeof(unsigned long long) * ((size_t)G + kSlots), s));
     int32_t* alive = reinterpret_cast<int32_t*>(sm + kSlotAlive);
     int32_t* bad = reinterpret_cast<int32_t*>(sm + kSlotBad);
     const int64_t N = h->lat.N;
-    const int64_t threads = (N + kSeg - 1) / kSeg;
     ::hp::count_launch();
-    k_counts<<<(unsigned)((threads + kT - 1) / kT), kT, 0, s>>>(h->q, N, G, h->m_counts, bad);
+    k_counts<<<counts_grid(N), kT, 0, s>>>(h->q, N, G, h->m_counts, bad);
     ::hp::count_launch();
-    k_alive<<<(G + kT - 1) / kT, kT, 0, s>>>(h->m_counts, G, alive);
-    if (orient) {
-        ::hp::count_launch();
-        k_bins<<<(G + kT - 1) / kT, kT, 0, s>>>(G, orient_kind, orient, h->m_bins);
-        ::hp::count_launch();
-        k_hist<<<(G + kT - 1) / kT, kT, 0, s>>>(G, orient_kind, h->m_bins, h->m_counts, sm + kSlotHist);
-    }
-    if (h->desc.field_mode == HP_FIELD_GRAIN) {
-        ::hp::count_launch();
-        k_field_sum_grain<<<(G + kT - 1) / kT, kT, 0, s>>>(h->m_counts, h->table, G, sm + kSlotField);
-    } else if (h->desc.field_mode == HP_FIELD_POINT) {
+    k_grain_stats<<<(G + kT - 1) / kT, kT, 0, s>>>(h->m_counts, G, orient_kind, orient,
+                                                   h->desc.field_mode == HP_FIELD_GRAIN ? h->table : nullptr,
+                                                   sm + kSlotHist, sm + kSlotField, alive);
+    if (h->desc.field_mode == HP_FIELD_POINT) {
         ::hp::count_launch();
         k_field_sum_point<<<4 * 152, kT, 0, s>>>(h->mp, h->table, (uint32_t)h->table_n, N, sm + kSlotField);
     }
