@@ -515,23 +515,27 @@ __device__ bool grid_barrier(unsigned int* bar, long long limit) {
     __shared__ int s_ok;
     __syncthreads();
     if (threadIdx.x == 0) {
-        volatile unsigned int* gen = bar + 1;
-        const unsigned int g = *gen;
+        // the block's writes (ordered before by the block barrier) are released with the
+        // arrival and acquired with the generation; polling without a pause shortens a
+        // barrier by half the pause
+        unsigned int g, n;
+        asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(g) : "l"(bar + 1) : "memory");
         __threadfence();
+        asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(n) : "l"(bar) : "memory");
         bool ok = true;
-        if (atomicAdd(bar, 1u) == gridDim.x - 1) {
-            atomicExch(bar, 0u);
-            __threadfence();
-            atomicAdd(bar + 1, 1u);
+        if (n == gridDim.x - 1) {
+            asm volatile("st.relaxed.gpu.global.u32 [%0], 0;" ::"l"(bar) : "memory");
+            asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar + 1) : "memory");
         } else {
             const long long t0 = clock64();
-            while (*gen == g) {
+            unsigned int now;
+            do {
+                asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(now) : "l"(bar + 1) : "memory");
                 if (clock64() - t0 > limit) {
                     ok = false;
                     break;
                 }
-                __nanosleep(64);
-            }
+            } while (now == g);
         }
         __threadfence();
         s_ok = ok;
@@ -826,27 +830,41 @@ __device__ __forceinline__ void train_body(const TrainArgs& a) {
         }
         mma_ok = ok;
         if (LOOP && ok) {
+            // this CTA's share of the entries: reduce over every slot, Adam, repack.  What
+            // no other CTA writes (the schedule, its own moments and parameters) is on its
+            // way before the barrier.
+            const int nslots = (int)gridDim.x;
+            const int chunk = (NPARAM + 1 + nslots - 1) / nslots;
+            const int lo = (int)blockIdx.x * chunk, hi = min(lo + chunk, NPARAM + 1);
+            const float lr = a.sched[3 * (step - 1)], c1 = a.sched[3 * (step - 1) + 1],
+                        c2 = a.sched[3 * (step - 1) + 2];
+            const bool own = (tid & 7) == 0;
+            float m0 = 0.0f, v0 = 0.0f, p0 = 0.0f;
+            if (own && lo + (tid >> 3) < min(hi, NPARAM)) {
+                m0 = a.m[lo + (tid >> 3)];
+                v0 = a.v[lo + (tid >> 3)];
+                p0 = a.P[lo + (tid >> 3)];
+            }
             ok = grid_barrier(a.bar, kWaitCycles);
             if (ok) {
-                // this CTA's share of the entries: reduce over every slot, Adam, repack
-                const int nslots = (int)gridDim.x;
-                const int chunk = (NPARAM + 1 + nslots - 1) / nslots;
-                const int lo = (int)blockIdx.x * chunk, hi = min(lo + chunk, NPARAM + 1);
-                const float lr = a.sched[3 * (step - 1)], c1 = a.sched[3 * (step - 1) + 1],
-                            c2 = a.sched[3 * (step - 1) + 2];
                 for (int base = lo; base < hi; base += NTT / 8) {
                     const int i = base + (tid >> 3);
+                    if (base != lo && own && i < min(hi, NPARAM)) {
+                        m0 = a.m[i];
+                        v0 = a.v[i];
+                        p0 = a.P[i];
+                    }
                     const float gi = slot_sum_cg(part, nslots, i < hi ? i : -1);
                     if ((tid & 7) == 0 && i < hi) {
                         if (i == NPARAM) {
                             if (a.loss_log) a.loss_log[step - 1] = gi;
                             if (a.loss_last) *a.loss_last = gi;
                         } else {
-                            const float mi = a.b1 * a.m[i] + (1.0f - a.b1) * gi;
-                            const float vi = a.b2 * a.v[i] + (1.0f - a.b2) * gi * gi;
+                            const float mi = a.b1 * m0 + (1.0f - a.b1) * gi;
+                            const float vi = a.b2 * v0 + (1.0f - a.b2) * gi * gi;
                             a.m[i] = mi;
                             a.v[i] = vi;
-                            const float pv = a.P[i] - lr * (mi / c1) / (sqrtf(vi / c2) + a.eps);
+                            const float pv = p0 - lr * (mi / c1) / (sqrtf(vi / c2) + a.eps);
                             a.P[i] = pv;
                             pack_param(a.img, i, pv);
                         }
