@@ -79,7 +79,6 @@ __host__ __device__ inline RMConsts rm_consts(double tau0, double taus, double h
 
 struct CPArgs {
     float C11, C12, C44;
-    double tau0, taus, h0;
     RMConsts rm;  // rm_consts(tau0, taus, h0), once per launch on the host
     double k;     // P:C:P, the same for every system of a cubic crystal
     Pair k2;
@@ -545,7 +544,6 @@ extern "C" int hp_cp_step(const hp_cp_params* prm, uint64_t seed, const int32_t*
     a.k = slip_stiffness(prm);
     a.k2 = pair_of(a.k);
     a.C11 = (float)prm->C11; a.C12 = (float)prm->C12; a.C44 = (float)prm->C44;
-    a.tau0 = prm->tau0; a.taus = prm->taus; a.h0 = prm->h0;
     a.rm = rm_consts(prm->tau0, prm->taus, prm->h0);
     a.beta = (float)prm->beta; a.G = (float)prm->G; a.e = (float)prm->e_incr; a.scale = (float)prm->energy_scale;
     a.w_weight = (float)prm->w_weight;
@@ -571,7 +569,6 @@ extern "C" int hp_cp_step_strain(const hp_cp_params* prm, uint64_t seed, const i
     a.k = slip_stiffness(prm);
     a.k2 = pair_of(a.k);
     a.C11 = (float)prm->C11; a.C12 = (float)prm->C12; a.C44 = (float)prm->C44;
-    a.tau0 = prm->tau0; a.taus = prm->taus; a.h0 = prm->h0;
     a.rm = rm_consts(prm->tau0, prm->taus, prm->h0);
     a.beta = (float)prm->beta; a.G = (float)prm->G; a.e = (float)prm->e_incr; a.scale = (float)prm->energy_scale;
     a.w_weight = (float)prm->w_weight;

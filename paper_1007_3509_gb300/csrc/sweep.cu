@@ -602,7 +602,6 @@ bool variant_ok(int nbr, int v, int field, bool m) {
 }
 
 bool variant_batch_ok(int nbr, int v, int field, bool m) {
-    const Variant var = variant_of(nbr, v);
     return variant_ok(nbr, v, field, m);
 }
 
@@ -636,7 +635,8 @@ PlaneArgs plane_args(const hp_handle* h, int variant, const int32_t* q_in, const
     a.tiles_x = (a.Lx + TX - 1) / TX;
     a.tiles = a.tiles_x * ((a.Ly + v.TY - 1) / v.TY);
     a.fast = (a.Lx >= v.WX && a.Ly >= WY) ? 1 : 0;
-    a.vec = (a.fast && (a.Lx % 4) == 0) ? 1 : 0;
+    const uintptr_t low = (uintptr_t)q_in | (uintptr_t)mp_in | (uintptr_t)q_nb | (uintptr_t)q_out | (uintptr_t)mp_out;
+    a.vec = (a.fast && (a.Lx % 4) == 0 && (low & 15u) == 0) ? 1 : 0;  // a caller's buffer may start on any int
     *planes = h->lat.nbr == 26 ? a.Lz / 2 : 1;
     return a;
 }

@@ -28,7 +28,7 @@ struct PlaneArgs {
     int tiles_x;
     int tiles;              // tiles per plane
     int fast;               // 1: window narrower than the lattice (wrap by one add)
-    int vec;                // 1: fast and Lx % 4 == 0 (16-byte row chunks)
+    int vec;                // 1: fast, Lx % 4 == 0 and every buffer on 16 bytes (16-byte row chunks)
     SweepKey key;           // what the draws of (seed, sweep) share
 };
 
