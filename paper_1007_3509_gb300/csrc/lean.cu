@@ -149,8 +149,8 @@ struct Lean {
     __device__ __forceinline__ int32_t mp_of(int pos, int o) const {
         if (o >= -(PS / 2) && o <= PS / 2) return MP[pos + o];
         const int n = pos + o + (o < 0 ? PS : -PS);
-        return __ldg(a.mp_nb + (o < 0 ? lobase : hibase) + (uint32_t)gx_of(n & (WX - 1)) +
-                     (uint32_t)a.Lx * (uint32_t)gy_of(n / WX));
+        return a.mp_nb[(o < 0 ? lobase : hibase) + (uint32_t)gx_of(n & (WX - 1)) +
+                       (uint32_t)a.Lx * (uint32_t)gy_of(n / WX)];
     }
     // The Metropolis test of the proposal at pos (offset o, acceptance draw u1).
     __device__ __forceinline__ void test(int pos, int o, uint32_t u1) const {
@@ -236,6 +236,9 @@ __device__ __forceinline__ void lean_body(const PlaneArgs& a, const LeanMaps* ma
         const int k = tid - 1, kk = k + (k >= 13);
         off[tid] = tid ? (kk / 9 - 1) * PS + ((kk / 3) % 3 - 1) * WX + (kk % 3 - 1) : 0;
     }
+    const bool chained = maps != nullptr, early = chained && chain_early();  // batched launches are not chained
+    if (early) chain_open();
+    if (chained) chain_wait();
     const uint32_t mb = s_addr(mbar);
     auto src = [&](int arr) -> const int32_t* {
         return arr == 0 ? a.q_nb + w.lobase : arr == 1 ? a.q_in + zbase : arr == 2 ? a.q_nb + w.hibase : a.mp_in + zbase;
@@ -362,6 +365,7 @@ __device__ __forceinline__ void lean_body(const PlaneArgs& a, const LeanMaps* ma
         if (p == 1) __syncthreads(); else __syncwarp();
     }
 
+    if (chained && !early) chain_open();
     // ---- write the warp's rows of the core: rows [2, WY - 2), columns [4, WX - 4)
     int32_t* qo = a.q_out + zbase;
     int32_t* mpo = HASMP ? a.mp_out + zbase : nullptr;
@@ -499,8 +503,8 @@ int launch_lean(const PlaneArgs& a, int planes, cudaStream_t s) {
         (uint64_t)a.Lx * a.Ly * a.Lz <= 0xFFFFFFFFull)
         maps.pf = encode_box(&maps.tab, a.table, a, WY) ? 1 : 0;
     count_launch();
-    k_lean26<WY, FIELD, HASMP><<<dim3((unsigned)a.tiles, (unsigned)planes), Cfg::kLT, smem, s>>>(a, maps);
-    HP_LAUNCH_CHECK("k_lean26");
+    HP_CUDA(launch_chained(k_lean26<WY, FIELD, HASMP>, dim3((unsigned)a.tiles, (unsigned)planes), Cfg::kLT, smem, s,
+                           a.chain != 0, a, maps));
     return HP_OK;
 }
 

@@ -630,6 +630,7 @@ PlaneArgs plane_args(const hp_handle* h, int variant, const int32_t* q_in, const
     a.Ly = (int)h->lat.L[1];
     a.Lz = (int)h->lat.L[2];
     a.zpar = zpar;
+    a.chain = 0;
     const Variant v = variant_of(h->lat.nbr, variant);
     const int TX = v.WX - 8, WY = window_rows(v);
     a.tiles_x = (a.Lx + TX - 1) / TX;
@@ -658,10 +659,10 @@ int plane_launch_batch(int nbr, int variant, int field, bool m, const PlaneArgs*
 // Variant a handle sweeps with until one is chosen (hp_set_sweep_variant or the
 // autotuner): the fastest measured on the benchmark lattices -- in 3D the lean
 // 64 x 32 window (512^3, grain field: 1.25e11 site-updates/s against 1.03e11 of
-// 64 x 44); in 2D the 128 x 28 lean tile (4 neighbours, 500^2 and 4096^2: 10.2 and
-// 61.6 us per MCS against 14.5 and 64.2 of 128 x 60; 8 neighbours, 1024^2: 12.7
-// against 16.8), but for 8 neighbours from 2048^2 sites on, where its halo costs
-// more than its latency saves, 128 x 60 (4096^2: 70.4 against 82.7).
+// 64 x 44); in 2D the 128 x 28 lean tile (4 neighbours, 500^2 and 3000^2: 6.8 and
+// 33.0 us per MCS against 11.6 and 39.0 of 128 x 60; 8 neighbours, 1024^2: 11.2
+// against 14.8), but for 8 neighbours from 2048^2 sites on, where its halo costs
+// more than its latency saves, 128 x 60 (24.2 against 25.3; 3000^2: 40.3 against 46.4).
 int default_variant(const hp_handle* h) {
     int v = 0;
     if (h->lat.nbr == 26) v = 11;
@@ -673,16 +674,17 @@ int default_variant(const hp_handle* h) {
 
 // Cluster size when these lattices are better swept by the resident 2D kernel, else
 // 0.  One lattice: 8 SMs at 0.1 us per MCS and 1000 sites against the tile
-// kernel's floor of 10 to 12 us a launch (300^2: 9.9 us per MCS against 10.3 and
-// 12.1 for 4 and 8 neighbours; 500^2: 18 against 10 and 12).  Several: the same
-// size each, or enough of them to fill the chip (8 neighbours, kT = 1, 100 MCS:
+// kernel's floor of 7 to 8 us a launch (220^2: 5.4 and 6.7 us per MCS for 4 and 8
+// neighbours against 7.0 and 8.2; 250^2, 6.1 and 6.7 against 10.0 and 11.1 without
+// 16-byte rows; 300^2: 9.9 against 6.8 and 7.9).  Several, whose launches cost 10 to
+// 12 us: up to 300^2 each, or enough of them to fill the chip (8 neighbours, kT = 1, 100 MCS:
 // 32 x 500^2 6.0 ms against 6.7, 100 x 500^2 14.0 against 19.5, but 4 x 500^2 2.0
 // against 1.6).
 int resident(hp_handle* const* m, int R) {
     int64_t sites = 0;
     for (int r = 0; r < R; ++r) sites += m[r]->lat.N;
     const int cs = res2d_cluster(m, R);
-    return cs && (sites <= (int64_t)R * 100000 || (int64_t)R * cs >= 152) ? cs : 0;
+    return cs && (sites <= (R == 1 ? 65536 : (int64_t)R * 100000) || (int64_t)R * cs >= 152) ? cs : 0;
 }
 
 int sweep_variants(int nbr) { return n_variants(nbr); }
@@ -724,13 +726,16 @@ int sweep_run(hp_handle* h, int32_t n_mcs, cudaStream_t s) {
         const uint32_t sw = (uint32_t)(h->sweep + t);
         int planes = 1, rc;
         if (nbr == 26) {
-            const PlaneArgs a0 = plane_args(h, v, qc, mc, qc, mc, qa, ma, sw, 0, &planes);
+            PlaneArgs a0 = plane_args(h, v, qc, mc, qc, mc, qa, ma, sw, 0, &planes);
+            a0.chain = t > 0;
             rc = plane_launch(h, v, a0, planes, s);
             if (rc) return rc;
-            const PlaneArgs a1 = plane_args(h, v, qc, mc, qa, ma, qa, ma, sw, 1, &planes);
+            PlaneArgs a1 = plane_args(h, v, qc, mc, qa, ma, qa, ma, sw, 1, &planes);
+            a1.chain = 1;
             rc = plane_launch(h, v, a1, planes, s);
         } else {
-            const PlaneArgs a0 = plane_args(h, v, qc, mc, nullptr, nullptr, qa, ma, sw, 0, &planes);
+            PlaneArgs a0 = plane_args(h, v, qc, mc, nullptr, nullptr, qa, ma, sw, 0, &planes);
+            a0.chain = t > 0;
             rc = h->an_J ? tile_launch_aniso(a0, aniso_of(h), h->desc.field_mode, m, nbr, s) : plane_launch(h, v, a0, planes, s);
         }
         if (rc) return rc;

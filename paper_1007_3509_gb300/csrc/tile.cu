@@ -116,8 +116,8 @@ struct Tile {
                 mpj = SMP[pos + off];
             } else {
                 const int r = pos / WX, col = pos - r * WX;
-                mpj = __ldg(a.mp_nb + wrap1(gx_of(col) + dx, a.Lx) + (int64_t)a.Lx * wrap1(gy_of(r) + dy, a.Ly) +
-                            sxy * (dz < 0 ? zlo : zhi));
+                mpj = a.mp_nb[wrap1(gx_of(col) + dx, a.Lx) + (int64_t)a.Lx * wrap1(gy_of(r) + dy, a.Ly) +
+                              sxy * (dz < 0 ? zlo : zhi)];
             }
         }
         if (FIELD == 1) { bi = tab(a.table, a.table_n, qi); bj = tab(a.table, a.table_n, qj); }
@@ -172,7 +172,7 @@ struct Tile {
 
 __device__ __forceinline__ bool al16(const void* p) { return ((uintptr_t)p & 15u) == 0; }
 
-template <int NBR, int WX, int WY, int FIELD, bool HASMP, bool ANI>
+template <int NBR, int WX, int WY, int FIELD, bool HASMP, bool ANI, bool CHAIN>
 __device__ __forceinline__ void tile_body(const PlaneArgs& a, const int tile, const int zidx, unsigned char* raw,
                                           const Aniso* an) {
     using T = Tile<NBR, WX, WY, FIELD, HASMP, ANI>;
@@ -211,6 +211,8 @@ __device__ __forceinline__ void tile_body(const PlaneArgs& a, const int tile, co
         return a.q_nb + sxy * (arr == Cfg::A_LO ? t.zlo : t.zhi);
     };
     if (threadIdx.x < 4) qn[threadIdx.x] = 0;
+    const bool early = CHAIN && chain_early();
+    if (early) chain_open();
     if (tma) {
         const uint32_t mb = s_addr(mbar);
         if (threadIdx.x == 0) {
@@ -218,6 +220,7 @@ __device__ __forceinline__ void tile_body(const PlaneArgs& a, const int tile, co
             asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         }
         __syncthreads();
+        if (CHAIN) chain_wait();
         if (threadIdx.x < 32) {
             if (threadIdx.x == 0)
                 asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(mb),
@@ -230,6 +233,7 @@ __device__ __forceinline__ void tile_body(const PlaneArgs& a, const int tile, co
         }
         if (!wait_or_drain(mb, &g_tile_err)) return;
     } else {
+        if (CHAIN) chain_wait();
         for (int i = threadIdx.x; i < ARR * WY * WX; i += kTileThreads) {
             const int arr = i / (WY * WX), rem = i - arr * (WY * WX), r = rem / WX, c = rem - r * WX;
             base[arr * AS + PAD + rem] = src(arr)[(int64_t)a.Lx * wrapi(t.y0 - Cfg::HY + r, a.Ly) + wrapi(t.x0 - 4 + c, a.Lx)];
@@ -393,6 +397,7 @@ __device__ __forceinline__ void tile_body(const PlaneArgs& a, const int tile, co
     }
     (void)M;
 
+    if (CHAIN && !early) chain_open();
     // ---- write the core: rows [HY, WY - HY), quads 1 .. QPR - 2 --------------
     int32_t* qo = a.q_out + sxy * t.z;
     int32_t* mpo = HASMP ? a.mp_out + sxy * t.z : nullptr;
@@ -420,14 +425,14 @@ __device__ __forceinline__ void tile_body(const PlaneArgs& a, const int tile, co
 template <int NBR, int WX, int WY, int FIELD, bool HASMP>
 __global__ void __launch_bounds__(kTileThreads, NBR == 26 ? 4 : 5) k_tile(const __grid_constant__ PlaneArgs a) {
     extern __shared__ __align__(16) unsigned char raw[];
-    tile_body<NBR, WX, WY, FIELD, HASMP, false>(a, (int)blockIdx.x, (int)blockIdx.y, raw, nullptr);
+    tile_body<NBR, WX, WY, FIELD, HASMP, false, true>(a, (int)blockIdx.x, (int)blockIdx.y, raw, nullptr);
 }
 
 template <int NBR, int WX, int WY, int FIELD, bool HASMP>
 __global__ void __launch_bounds__(kTileThreads, 5)
     k_tile_aniso(const __grid_constant__ PlaneArgs a, const __grid_constant__ Aniso an) {
     extern __shared__ __align__(16) unsigned char raw[];
-    tile_body<NBR, WX, WY, FIELD, HASMP, true>(a, (int)blockIdx.x, 0, raw, &an);
+    tile_body<NBR, WX, WY, FIELD, HASMP, true, true>(a, (int)blockIdx.x, 0, raw, &an);
 }
 
 // Many independent lattices in one launch: block b belongs to the replica r
@@ -453,7 +458,7 @@ __global__ void __launch_bounds__(kTileThreads, NBR == 26 ? 4 : 5)
         s_tile = (int)(local - (int64_t)s_zidx * sa.tiles);
     }
     __syncthreads();
-    tile_body<NBR, WX, WY, FIELD, HASMP, false>(sa, s_tile, s_zidx, raw, nullptr);
+    tile_body<NBR, WX, WY, FIELD, HASMP, false, false>(sa, s_tile, s_zidx, raw, nullptr);
 }
 
 struct TileBatch {
@@ -479,7 +484,8 @@ int launch_tile(const PlaneArgs* a, const TileBatch* b, int planes, cudaStream_t
     if (a) {
         if (a->tiles == 0) return HP_OK;
         count_launch();
-        k_tile<NBR, WX, WY, FIELD, HASMP><<<dim3((unsigned)a->tiles, (unsigned)planes), kTileThreads, smem, s>>>(*a);
+        HP_CUDA(launch_chained(k_tile<NBR, WX, WY, FIELD, HASMP>, dim3((unsigned)a->tiles, (unsigned)planes), kTileThreads,
+                               smem, s, a->chain != 0, *a));
     } else {
         if (b->blocks == 0) return HP_OK;  // configure only
         count_launch();
@@ -522,14 +528,14 @@ int launch_aniso(const PlaneArgs& a, const Aniso& an, cudaStream_t s) {
     HP_CUDA(cudaFuncSetAttribute(k_tile_aniso<NBR, 128, 32, FIELD, HASMP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)smem));
     count_launch();
-    k_tile_aniso<NBR, 128, 32, FIELD, HASMP><<<(unsigned)a.tiles, kTileThreads, smem, s>>>(a, an);
-    HP_LAUNCH_CHECK("k_tile_aniso");
+    HP_CUDA(launch_chained(k_tile_aniso<NBR, 128, 32, FIELD, HASMP>, dim3((unsigned)a.tiles), kTileThreads, smem, s,
+                           a.chain != 0, a, an));
     return HP_OK;
 }
 
 }  // namespace
 
-// 1024^2, 8 neighbours, Read-Shockley tables: 20.7 us per MCS; 72 us on the per-colour
+// 1024^2, 8 neighbours, Read-Shockley tables: 18.7 us per MCS; 72 us on the per-colour
 // kernel, four launches whose bins took a 64-bit remainder and division each.
 int tile_launch_aniso(const PlaneArgs& a, const Aniso& an, int field, bool hasmp, int nbr, cudaStream_t s) {
     if (field == HP_FIELD_POINT && hasmp) return nbr == 8 ? launch_aniso<8, 2, true>(a, an, s) : launch_aniso<4, 2, true>(a, an, s);
