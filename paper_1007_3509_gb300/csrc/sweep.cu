@@ -49,6 +49,9 @@ struct PhaseArgs {
 // One colour phase, one thread per site of that colour, in place.
 // FIELD: 0 none, 1 grain (table[q]), 2 point (table[mp]).
 // ---------------------------------------------------------------------------
+// A small lattice is bound by the launches, one per colour, which are chained (3D, 6
+// neighbours: 64^3, 20 MCS 179 -> 112 us; 128^3 586 -> 459; 250 x 200 x 130, 10 MCS
+// 670 -> 628; 400^3 alike).
 // ANI: the energy of a site in state s is the sum over neighbours n with
 // q_n != s of jtab[bin(s, q_n)], and the Metropolis threshold is scaled by the
 // mobility of the (q_i, q_j) boundary (metropolis_mob).
@@ -85,6 +88,8 @@ __global__ void __launch_bounds__(kThreads) k_phase(const __grid_constant__ Phas
         yc[d] = (uint32_t)a.Lx * (uint32_t)wrap1(y + d - 1, a.Ly);
         zc[d] = DIM == 3 ? sxy * (uint32_t)wrap1(z + d - 1, a.Lz) : 0u;
     }
+    chain_open();
+    chain_wait();
     const int32_t qi = a.q[i];
     int32_t nv[G::M];
     int same_old = 0;
@@ -446,7 +451,7 @@ __global__ void __launch_bounds__(kThreads, kPlaneMinBlocks) k_plane_batch(Batch
 }
 
 template <int DIM, int NBR, int FIELD, bool HASMP, bool ANI>
-int launch_phase(hp_handle* h, uint32_t sweep, int colour, cudaStream_t s) {
+int launch_phase(hp_handle* h, uint32_t sweep, int colour, bool chain, cudaStream_t s) {
     PhaseArgs a;
     a.q = h->q;
     a.mp = h->mp;
@@ -466,38 +471,37 @@ int launch_phase(hp_handle* h, uint32_t sweep, int colour, cudaStream_t s) {
     a.an = aniso_of(h);
     const int64_t blocks = ((int64_t)a.n_colour_sites + kThreads - 1) / kThreads;
     ::hp::count_launch();
-    k_phase<DIM, NBR, FIELD, HASMP, ANI><<<(unsigned)blocks, kThreads, 0, s>>>(a);
-    HP_LAUNCH_CHECK("k_phase");
+    HP_CUDA(launch_chained(k_phase<DIM, NBR, FIELD, HASMP, ANI>, dim3((unsigned)blocks), kThreads, 0, s, chain, a));
     return HP_OK;
 }
 
 template <int DIM, int NBR, bool ANI>
-int phase_dispatch_a(hp_handle* h, uint32_t sweep, int colour, cudaStream_t s) {
+int phase_dispatch_a(hp_handle* h, uint32_t sweep, int colour, bool chain, cudaStream_t s) {
     const bool m = h->mp != nullptr;
     switch (h->desc.field_mode) {
         case HP_FIELD_NONE:
-            return m ? launch_phase<DIM, NBR, 0, true, ANI>(h, sweep, colour, s)
-                     : launch_phase<DIM, NBR, 0, false, ANI>(h, sweep, colour, s);
+            return m ? launch_phase<DIM, NBR, 0, true, ANI>(h, sweep, colour, chain, s)
+                     : launch_phase<DIM, NBR, 0, false, ANI>(h, sweep, colour, chain, s);
         case HP_FIELD_GRAIN:
-            return m ? launch_phase<DIM, NBR, 1, true, ANI>(h, sweep, colour, s)
-                     : launch_phase<DIM, NBR, 1, false, ANI>(h, sweep, colour, s);
+            return m ? launch_phase<DIM, NBR, 1, true, ANI>(h, sweep, colour, chain, s)
+                     : launch_phase<DIM, NBR, 1, false, ANI>(h, sweep, colour, chain, s);
         default:
-            return launch_phase<DIM, NBR, 2, true, ANI>(h, sweep, colour, s);
+            return launch_phase<DIM, NBR, 2, true, ANI>(h, sweep, colour, chain, s);
     }
 }
 
 template <int DIM, int NBR>
-int phase_dispatch(hp_handle* h, uint32_t sweep, int colour, cudaStream_t s) {
-    return h->an_J ? phase_dispatch_a<DIM, NBR, true>(h, sweep, colour, s)
-                   : phase_dispatch_a<DIM, NBR, false>(h, sweep, colour, s);
+int phase_dispatch(hp_handle* h, uint32_t sweep, int colour, bool chain, cudaStream_t s) {
+    return h->an_J ? phase_dispatch_a<DIM, NBR, true>(h, sweep, colour, chain, s)
+                   : phase_dispatch_a<DIM, NBR, false>(h, sweep, colour, chain, s);
 }
 
-int run_phase_kernel(hp_handle* h, uint32_t sweep, int colour, cudaStream_t s) {
+int run_phase_kernel(hp_handle* h, uint32_t sweep, int colour, bool chain, cudaStream_t s) {
     const int dim = h->lat.dim, nbr = h->lat.nbr;
-    if (dim == 2 && nbr == 4) return phase_dispatch<2, 4>(h, sweep, colour, s);
-    if (dim == 2 && nbr == 8) return phase_dispatch<2, 8>(h, sweep, colour, s);
-    if (dim == 3 && nbr == 6) return phase_dispatch<3, 6>(h, sweep, colour, s);
-    return phase_dispatch<3, 26>(h, sweep, colour, s);
+    if (dim == 2 && nbr == 4) return phase_dispatch<2, 4>(h, sweep, colour, chain, s);
+    if (dim == 2 && nbr == 8) return phase_dispatch<2, 8>(h, sweep, colour, chain, s);
+    if (dim == 3 && nbr == 6) return phase_dispatch<3, 6>(h, sweep, colour, chain, s);
+    return phase_dispatch<3, 26>(h, sweep, colour, chain, s);
 }
 
 // Tile variants of the fused kernel.  Plane tiles (this file): window width WX
@@ -703,7 +707,7 @@ int sweep_run(hp_handle* h, int32_t n_mcs, cudaStream_t s) {
     if (!fused) {
         for (int32_t t = 0; t < n_mcs; ++t)
             for (int c = 0; c < h->lat.colours; ++c) {
-                const int rc = run_phase_kernel(h, (uint32_t)(h->sweep + t), c, s);
+                const int rc = run_phase_kernel(h, (uint32_t)(h->sweep + t), c, t + c > 0, s);
                 if (rc) return rc;
             }
         h->sweep += (uint64_t)n_mcs;
