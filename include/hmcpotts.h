@@ -58,7 +58,7 @@ extern "C" {
                           /* HP_ORIENT_ANGLE angle t about z (Sec. 5), float[4G]     */
 
 /* Sweep kernel choice (hp_set_sweep_kernel). */
-#define HP_SWEEP_AUTO 0   /* fused multi-phase tiles where available            */
+#define HP_SWEEP_AUTO 0   /* the route measured fastest for the lattice       */
 #define HP_SWEEP_PHASE 1  /* one launch per colour phase, in place              */
 #define HP_SWEEP_FUSED 2  /* all phases of a plane in shared memory, double-buffered */
 

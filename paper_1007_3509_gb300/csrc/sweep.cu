@@ -677,18 +677,29 @@ int default_variant(const hp_handle* h) {
 }
 
 // Cluster size when these lattices are better swept by the resident 2D kernel, else
-// 0.  One lattice: 8 SMs at 0.1 us per MCS and 1000 sites against the tile
-// kernel's floor of 7 to 8 us a launch (220^2: 5.4 and 6.7 us per MCS for 4 and 8
-// neighbours against 7.0 and 8.2; 250^2, 6.1 and 6.7 against 10.0 and 11.1 without
-// 16-byte rows; 300^2: 9.9 against 6.8 and 7.9).  Several, whose launches cost 10 to
-// 12 us: up to 300^2 each, or enough of them to fill the chip (8 neighbours, kT = 1, 100 MCS:
-// 32 x 500^2 6.0 ms against 6.7, 100 x 500^2 14.0 against 19.5, but 4 x 500^2 2.0
-// against 1.6).
+// 0.  One lattice, 8 neighbours: 8 SMs at 0.1 us per MCS and 1000 sites against the
+// tile kernel's floor of 7 to 8 us a launch (220^2: 6.7 us per MCS against 8.2; 250^2,
+// 6.7 against 11.1 without 16-byte rows; 300^2: 9.9 against 7.9).  4 neighbours: against
+// the per-colour kernel's 3.7 us per MCS (128^2, rows of one pass of a warp: 2.9;
+// 136^2: 4.3).  Several, whose launches cost 10 to 12 us: up to 300^2 each, or enough of
+// them to fill the chip (8 neighbours, kT = 1, 100 MCS: 32 x 500^2 6.0 ms against 6.7,
+// 100 x 500^2 14.0 against 19.5, but 4 x 500^2 2.0 against 1.6).
 int resident(hp_handle* const* m, int R) {
     int64_t sites = 0;
     for (int r = 0; r < R; ++r) sites += m[r]->lat.N;
     const int cs = res2d_cluster(m, R);
-    return cs && (sites <= (R == 1 ? 65536 : (int64_t)R * 100000) || (int64_t)R * cs >= 152) ? cs : 0;
+    const int64_t most = R > 1 ? 100000 : m[0]->lat.nbr == 4 ? 16384 : 65536;
+    return cs && (sites <= R * most || (int64_t)R * cs >= 152) ? cs : 0;
+}
+
+// Lattices that the per-colour kernel sweeps faster than the fused one: two chained
+// launches of one site a thread against a window's fill and halo.  us per MCS, 50 and
+// 500 sites a grain: 256^2 3.8 and 3.8 against 8.4 and 6.8, 700^2 5.9 and 5.7 against 8.5
+// and 6.9, with material points 6.6 and 6.4 against 11.0 and 9.3; 1500^2 18.0 and 17.5
+// against 15.3 and 11.1.  With misorientation tables 300^2 9.4 and 7.5 against 13.0 and
+// 9.0, 360^2 11.5 and 10.0 against 13.0 and 9.0.
+bool per_colour(const hp_handle* h) {
+    return h->lat.nbr == 4 && h->lat.N < (h->an_J ? 100000 : (int64_t)1 << 19);
 }
 
 int sweep_variants(int nbr) { return n_variants(nbr); }
@@ -703,7 +714,17 @@ int sweep_run(hp_handle* h, int32_t n_mcs, cudaStream_t s) {
     // built, the others on the per-colour kernel
     const bool tiles = h->an_J && h->lat.dim == 2 &&
                        (h->mp ? h->desc.field_mode == HP_FIELD_POINT : h->desc.field_mode != HP_FIELD_POINT);
-    const bool fused = nbr != 6 && (!h->an_J || tiles) && h->sweep_kernel != HP_SWEEP_PHASE;
+    bool fused = nbr != 6 && (!h->an_J || tiles) && h->sweep_kernel != HP_SWEEP_PHASE;
+    if (fused && h->sweep_kernel == HP_SWEEP_AUTO && h->sweep_variant < 0) {
+        const int cs = resident(&h, 1);
+        if (cs) {
+            const int rc = res2d_run(&h, 1, cs, n_mcs, s);
+            if (rc) return rc;
+            h->sweep += (uint64_t)n_mcs;
+            return HP_OK;
+        }
+        fused = !per_colour(h);
+    }
     if (!fused) {
         for (int32_t t = 0; t < n_mcs; ++t)
             for (int c = 0; c < h->lat.colours; ++c) {
@@ -712,15 +733,6 @@ int sweep_run(hp_handle* h, int32_t n_mcs, cudaStream_t s) {
             }
         h->sweep += (uint64_t)n_mcs;
         return HP_OK;
-    }
-    if (h->sweep_kernel == HP_SWEEP_AUTO && h->sweep_variant < 0) {
-        const int cs = resident(&h, 1);
-        if (cs) {
-            const int rc = res2d_run(&h, 1, cs, n_mcs, s);
-            if (rc) return rc;
-            h->sweep += (uint64_t)n_mcs;
-            return HP_OK;
-        }
     }
     const bool m = h->mp != nullptr;
     const int v = h->an_J ? kAnisoVariant : h->sweep_variant >= 0 ? h->sweep_variant : default_variant(h);
