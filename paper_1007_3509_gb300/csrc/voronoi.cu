@@ -25,6 +25,7 @@
 
 
 #include "common.cuh"
+#include "reach.h"
 
 namespace hp {
 namespace {
@@ -165,22 +166,6 @@ __global__ void __launch_bounds__(kT) k_assign(int32_t* q, int32_t* mp, int64_t 
     if (mp) mp[i] = (int32_t)i;
 }
 
-// Least and largest periodic distance of coordinate s to the interval [b, b + len] of
-// an axis of (even, or 1) length L > len.
-struct Reach {
-    int lo, hi;
-};
-__device__ __forceinline__ Reach reach(int s, int b, int len, int L) {
-    int u = s - b;
-    u += u < 0 ? L : 0;  // 0 <= u < L
-    const int v = u > len ? u - len : len - u;
-    int h = u + (L >> 1);
-    h -= h >= L ? L : 0;  // offset of the point opposite to s
-    Reach r;
-    r.lo = u <= len ? 0 : min(u - len, L - u);
-    r.hi = h <= len ? L >> 1 : max(min(u, L - u), min(v, L - v));
-    return r;
-}
 struct Box {
     int b[3], len[3];
 };
@@ -195,7 +180,8 @@ __device__ __forceinline__ Reach reach2(const int4 s, const Box& k, const Cells&
 // to a lane: compact, for a short list, and 32 bytes of a row, for whole sectors.
 // kNear seeds per brick and kRun per run; beyond, a run tests the brick's list and a
 // brick its sites' own rings.  256^3, 16000 seeds, whole call: 3.1 ms with the rings
-// per site.
+// per site, 0.34 ms with bricks (0.45 ms while a run's upper bound exceeded the largest
+// distance by its length and some 25 seeds of a run's list stood for six).
 constexpr int kNear = 1024, kRun = 64;
 
 template <int DIM>
@@ -221,12 +207,8 @@ __device__ __forceinline__ void brick_runs(const Box& k, const Cells& c, const i
         m.b[2] = k.b[2] + (t / (B::NX * B::NY)) * B::RZ;
         if (m.b[0] >= c.L[0] || m.b[1] >= c.L[1] || m.b[2] >= c.L[2]) continue;
         const int full[3] = {B::RX, B::RY, B::RZ};
-        int end[3];
 #pragma unroll
-        for (int d = 0; d < 3; ++d) {
-            m.len[d] = min(full[d], c.L[d] - m.b[d]) - 1;
-            end[d] = m.b[d] + m.len[d];
-        }
+        for (int d = 0; d < 3; ++d) m.len[d] = min(full[d], c.L[d] - m.b[d]) - 1;
         auto reach_of = [&](const int4 s) {
             if (!NEAR) return reach2(s, m, c);
             const int sd[3] = {s.x, s.y, s.z};
@@ -234,10 +216,9 @@ __device__ __forceinline__ void brick_runs(const Box& k, const Cells& c, const i
 #pragma unroll
             for (int d = 0; d < 3; ++d) {
                 if (DIM == 2 && d == 2) continue;
-                const int u = m.b[d] - sd[d], v = sd[d] - end[d];  // past either end
-                const int lo = max(max(u, v), 0), hi = m.len[d] - min(u, v);
-                r.lo += lo * lo;
-                r.hi += hi * hi;
+                const Reach a = reach_near(sd[d], m.b[d], m.len[d]);
+                r.lo += a.lo * a.lo;
+                r.hi += a.hi * a.hi;
             }
             return r;
         };
