@@ -118,8 +118,8 @@ __device__ __forceinline__ int wrapc(int a, int n) {
     return a < 0 ? a + n : a;
 }
 
-// Nearest seed of one site by its own rings of cells: what a brick with too many
-// seeds nearby, and lattices too long for 32-bit distances, fall back to.
+// Nearest seed of one site by its own rings of cells: for lattices that are not
+// assigned by bricks, and for a brick with more seeds nearby than its list holds.
 __device__ __noinline__ int32_t assign_site(int x, int y, int z, const Cells& c, const int32_t* start, const int4* list) {
     const int cx = cell_of(x, c.L[0], c.nc[0]), cy = cell_of(y, c.L[1], c.nc[1]), cz = cell_of(z, c.L[2], c.nc[2]);
     int64_t best = INT64_MAX;
@@ -182,11 +182,12 @@ __device__ __forceinline__ Reach reach2(const int4 s, const Box& k, const Cells&
 // brick its sites' own rings.  256^3, 16000 seeds, whole call: 3.1 ms with the rings
 // per site, 0.34 ms with bricks (0.45 ms while a run's upper bound exceeded the largest
 // distance by its length and some 25 seeds of a run's list stood for six).
-constexpr int kNear = 1024, kRun = 64;
+constexpr int kRun = 64;
 
 template <int DIM>
 struct Brick {
-    static constexpr int X = DIM == 3 ? 32 : 64, Y = DIM == 3 ? 8 : 32, Z = DIM == 3 ? 8 : 1;
+    static constexpr int X = DIM == 3 ? kBrick3[0] : kBrick2[0], Y = DIM == 3 ? kBrick3[1] : kBrick2[1],
+                         Z = DIM == 3 ? kBrick3[2] : kBrick2[2];
     static constexpr int RX = 8, RY = DIM == 3 ? 4 : 8, RZ = DIM == 3 ? 2 : 1;  // lanes: 8 x 4, twice (in z; in y)
     static constexpr int NX = X / RX, NY = Y / RY, RUNS = NX * NY * (Z / RZ);
 };
@@ -387,12 +388,11 @@ __global__ void __launch_bounds__(kT) k_assign_bricks(int32_t* __restrict__ q, i
     }
 }
 
-// Bricks where squared distances stay below 2^31 (axes up to 32768), single sites
-// otherwise.
-void launch_assign(int32_t* q, int32_t* mp, int64_t N, const Cells& c, const int32_t* start, const int4* list,
+// Bricks or single sites, see assign_by_bricks.
+void launch_assign(int32_t* q, int32_t* mp, int64_t N, const Cells& c, int32_t G, const int32_t* start, const int4* list,
                    cudaStream_t s) {
     ::hp::count_launch();
-    if (c.L[0] > 32768 || c.L[1] > 32768 || c.L[2] > 32768) {
+    if (!assign_by_bricks(c.dim, c.L, G)) {
         k_assign<<<(unsigned)((N + kT - 1) / kT), kT, 0, s>>>(q, mp, N, c, start, list);
     } else if (c.dim == 3) {
         using B = Brick<3>;
@@ -506,7 +506,7 @@ int voronoi_run(hp_handle* h, int32_t orient_kind, float* orient, int64_t* seed_
         k_scan<<<1, 1024, 0, s>>>(cnt, start, (int32_t)ncell);
         ::hp::count_launch();
         k_cell_scatter<<<gb, kT, 0, s>>>(xyz, G, start, cursor, list);
-        launch_assign(h->q, h->mp, N, c, start, list, s);
+        launch_assign(h->q, h->mp, N, c, G, start, list, s);
         if ((e = cudaGetLastError())) break;
         if (orient) {
             ::hp::count_launch();
@@ -635,7 +635,7 @@ extern "C" int hp_init_voronoi_static(hp_handle* h, int32_t orient_kind, float* 
     k_scan<<<1, 1024, 0, s>>>(cnt, start, (int32_t)ncell);
     ::hp::count_launch();
     k_cell_scatter<<<gb, kT, 0, s>>>(xyz, G, start, cursor, list);
-    launch_assign(h->q, h->mp, N, c, start, list, s);
+    launch_assign(h->q, h->mp, N, c, G, start, list, s);
     if (orient) {
         ::hp::count_launch();
         k_orient<<<gb, kT, 0, s>>>(G, h->desc.seed, orient_kind, orient);
