@@ -26,7 +26,8 @@
 //  * four warps of WY / 8 row pairs each: about 28 of the 128 sites a warp looks
 //    at per phase go on to its test, one per lane, so a pass runs nearly full.
 //    With eight warps (14 proposals, two lanes to each) the same window took 66 %
-//    more instructions and 138 us where this takes 100;
+//    more instructions and 138 us where this takes 100.  A launch of few windows
+//    waits rather than issues and takes eight (lean_warps);
 //  * the neighbour planes' material points are gathered for the proposals that
 //    point there instead of being staged: 37 KB of shared memory a block, six
 //    blocks on an SM (staged, 53 KB and four).
@@ -38,6 +39,7 @@
 
 #include <cudaTypedefs.h>
 
+#include "routes.h"
 #include "sweep.cuh"
 
 namespace hp {
@@ -70,9 +72,9 @@ __device__ __forceinline__ void tma_prefetch_l2(const CUtensorMap* map, int x, i
 }
 
 
-template <int WY, int FIELD, bool HASMP>
+template <int WY, int FIELD, bool HASMP, int NW_ = 4>
 struct LeanCfg {
-    static constexpr int NW = 4, kLT = 32 * NW;
+    static constexpr int NW = NW_, kLT = 32 * NW;
     static constexpr int WX = 64, HX = 4, HY = 2, TX = WX - 2 * HX, TY = WY - 2 * HY;
     static constexpr int PS = WX * WY;             // one plane window, sites
     static constexpr int NA = HASMP ? 4 : 3;       // window arrays: q(z-1) q(z) q(z+1) [mp(z)]
@@ -88,7 +90,7 @@ struct LeanCfg {
     static constexpr size_t smem() { return 128 + 4 * (size_t)NA * PS + 8 * (size_t)(NW * CAP) + 4 * 28 + 8; }
     // blocks per SM that the shared memory allows (228 KB, 1 KB of it per block taken)
     static constexpr int FIT = (int)(228 * 1024 / (smem() + 1024));
-    static constexpr int MINB = FIT > 7 ? 7 : FIT;
+    static constexpr int MINB = NW > 4 ? 3 : FIT > 7 ? 7 : FIT;
     __host__ __device__ static constexpr int ylo(int p) { return 1 + (p >> 1); }
 };
 
@@ -118,9 +120,9 @@ __device__ __noinline__ int wrap_any(int a, int L) { return wrapi(a, L); }
 
 // One window (tile `tile` of plane 2 zidx + a.zpar) of one lattice; maps NULL
 // when no window of this launch is copied by TMA boxes.
-template <int WY, int FIELD, bool HASMP>
+template <int WY, int FIELD, bool HASMP, int NW>
 struct Lean {
-    using Cfg = LeanCfg<WY, FIELD, HASMP>;
+    using Cfg = LeanCfg<WY, FIELD, HASMP, NW>;
     static constexpr int WX = Cfg::WX, PS = Cfg::PS;
     const PlaneArgs& a;
     int32_t* Q;         // q of plane z (z-1 at -PS, z+1 at +PS)
@@ -189,13 +191,13 @@ struct Lean {
     }
 };
 
-template <int WY, int FIELD, bool HASMP>
+template <int WY, int FIELD, bool HASMP, int NW>
 __device__ __forceinline__ void lean_body(const PlaneArgs& a, const LeanMaps* maps, const int tile, const int zidx,
                                           unsigned char* raw) {
-    using L = Lean<WY, FIELD, HASMP>;
+    using L = Lean<WY, FIELD, HASMP, NW>;
     using Cfg = typename L::Cfg;
     constexpr int WX = Cfg::WX, PS = Cfg::PS, NA = Cfg::NA, PER = Cfg::PER, CAP = Cfg::CAP;
-    constexpr int NW = Cfg::NW, kLT = Cfg::kLT;
+    constexpr int kLT = Cfg::kLT;
     constexpr bool EVEN = Cfg::SY % NW == 0;  // every warp has PER row pairs
     int32_t* base = reinterpret_cast<int32_t*>(raw + ((128u - (s_addr(raw) & 127u)) & 127u));
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -403,18 +405,18 @@ __device__ __forceinline__ void lean_body(const PlaneArgs& a, const LeanMaps* ma
     }
 }
 
-template <int WY, int FIELD, bool HASMP>
-__global__ void __launch_bounds__(LeanCfg<WY, FIELD, HASMP>::kLT, LeanCfg<WY, FIELD, HASMP>::MINB)
+template <int WY, int FIELD, bool HASMP, int NW>
+__global__ void __launch_bounds__(LeanCfg<WY, FIELD, HASMP, NW>::kLT, LeanCfg<WY, FIELD, HASMP, NW>::MINB)
     k_lean26(const __grid_constant__ PlaneArgs a, const __grid_constant__ LeanMaps maps) {
     extern __shared__ __align__(16) unsigned char raw[];
-    lean_body<WY, FIELD, HASMP>(a, &maps, (int)blockIdx.x, (int)blockIdx.y, raw);
+    lean_body<WY, FIELD, HASMP, NW>(a, &maps, (int)blockIdx.x, (int)blockIdx.y, raw);
 }
 
 // Many independent lattices in one launch: block b belongs to the replica r
 // with start[r] <= b < start[r+1]; within it b - start[r] = zidx * tiles + tile.
 // Windows are filled by the asynchronous 16-byte copies.
-template <int WY, int FIELD, bool HASMP>
-__global__ void __launch_bounds__(LeanCfg<WY, FIELD, HASMP>::kLT, LeanCfg<WY, FIELD, HASMP>::MINB)
+template <int WY, int FIELD, bool HASMP, int NW>
+__global__ void __launch_bounds__(LeanCfg<WY, FIELD, HASMP, NW>::kLT, LeanCfg<WY, FIELD, HASMP, NW>::MINB)
     k_lean26_batch(const PlaneArgs* __restrict__ args, const int64_t* __restrict__ start, int R, uint32_t sweep_add) {
     extern __shared__ __align__(16) unsigned char raw[];
     __shared__ PlaneArgs sa;
@@ -434,7 +436,7 @@ __global__ void __launch_bounds__(LeanCfg<WY, FIELD, HASMP>::kLT, LeanCfg<WY, FI
         s_tile = (int)(local - (int64_t)s_zidx * sa.tiles);
     }
     __syncthreads();
-    lean_body<WY, FIELD, HASMP>(sa, nullptr, s_tile, s_zidx, raw);
+    lean_body<WY, FIELD, HASMP, NW>(sa, nullptr, s_tile, s_zidx, raw);
 }
 
 PFN_cuTensorMapEncodeTiled_v12000 map_encoder() {
@@ -467,30 +469,16 @@ bool encode_box(CUtensorMap* m, const void* base, const PlaneArgs& a, int WY) {
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// Opt both kernels of an instantiation into their dynamic shared memory, once.
-template <int WY, int FIELD, bool HASMP>
-int lean_configure(size_t smem) {
-    static bool configured = false;
+template <int WY, int FIELD, bool HASMP, int NW>
+int launch_lean_nw(const PlaneArgs& a, int planes, cudaStream_t s) {
+    using Cfg = LeanCfg<WY, FIELD, HASMP, NW>;
+    constexpr size_t smem = Cfg::smem();
+    static bool configured = false;  // per template instance
     if (!configured) {
-        HP_CUDA(cudaFuncSetAttribute(k_lean26<WY, FIELD, HASMP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)smem));
-        HP_CUDA(cudaFuncSetAttribute(k_lean26_batch<WY, FIELD, HASMP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        HP_CUDA(cudaFuncSetAttribute(k_lean26<WY, FIELD, HASMP, NW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)smem));
         configured = true;
     }
-    return HP_OK;
-}
-#define HP_CUDA_ONCE_ATTR(WY_, F_, M_, SM_)                   \
-    do {                                                      \
-        const int rc_ = lean_configure<WY_, F_, M_>(SM_);     \
-        if (rc_) return rc_;                                  \
-    } while (0)
-
-template <int WY, int FIELD, bool HASMP>
-int launch_lean(const PlaneArgs& a, int planes, cudaStream_t s) {
-    using Cfg = LeanCfg<WY, FIELD, HASMP>;
-    constexpr size_t smem = Cfg::smem();
-    HP_CUDA_ONCE_ATTR(WY, FIELD, HASMP, smem);
     if (a.tiles == 0 || planes == 0) return HP_OK;
     LeanMaps maps;
     memset(&maps, 0, sizeof(maps));
@@ -503,22 +491,48 @@ int launch_lean(const PlaneArgs& a, int planes, cudaStream_t s) {
         (uint64_t)a.Lx * a.Ly * a.Lz <= 0xFFFFFFFFull)
         maps.pf = encode_box(&maps.tab, a.table, a, WY) ? 1 : 0;
     count_launch();
-    HP_CUDA(launch_chained(k_lean26<WY, FIELD, HASMP>, dim3((unsigned)a.tiles, (unsigned)planes), Cfg::kLT, smem, s,
+    HP_CUDA(launch_chained(k_lean26<WY, FIELD, HASMP, NW>, dim3((unsigned)a.tiles, (unsigned)planes), Cfg::kLT, smem, s,
                            a.chain != 0, a, maps));
+    return HP_OK;
+}
+
+template <int WY, int FIELD, bool HASMP>
+int launch_lean(const PlaneArgs& a, int planes, cudaStream_t s) {
+    if constexpr (HASMP && WY == 32)
+        if (lean_warps((int64_t)a.tiles * planes) == 8) return launch_lean_nw<WY, FIELD, HASMP, 8>(a, planes, s);
+    return launch_lean_nw<WY, FIELD, HASMP, 4>(a, planes, s);
+}
+
+template <int WY, int FIELD, bool HASMP, int NW>
+int launch_lean_batch_nw(const PlaneArgs* d_args, const int64_t* d_start, int R, int64_t blocks, uint32_t sweep_add,
+                         cudaStream_t s) {
+    using Cfg = LeanCfg<WY, FIELD, HASMP, NW>;
+    constexpr size_t smem = Cfg::smem();
+    static bool configured = false;  // per template instance
+    if (!configured) {
+        HP_CUDA(cudaFuncSetAttribute(k_lean26_batch<WY, FIELD, HASMP, NW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)smem));
+        configured = true;
+    }
+    if (blocks == 0) return HP_OK;  // configure only (outside a graph capture)
+    count_launch();
+    k_lean26_batch<WY, FIELD, HASMP, NW><<<(unsigned)blocks, Cfg::kLT, smem, s>>>(d_args, d_start, R, sweep_add);
+    HP_LAUNCH_CHECK("k_lean26_batch");
     return HP_OK;
 }
 
 template <int WY, int FIELD, bool HASMP>
 int launch_lean_batch(const PlaneArgs* d_args, const int64_t* d_start, int R, int64_t blocks, uint32_t sweep_add,
                       cudaStream_t s) {
-    using Cfg = LeanCfg<WY, FIELD, HASMP>;
-    constexpr size_t smem = Cfg::smem();
-    HP_CUDA_ONCE_ATTR(WY, FIELD, HASMP, smem);
-    if (blocks == 0) return HP_OK;  // configure only (outside a graph capture)
-    count_launch();
-    k_lean26_batch<WY, FIELD, HASMP><<<(unsigned)blocks, Cfg::kLT, smem, s>>>(d_args, d_start, R, sweep_add);
-    HP_LAUNCH_CHECK("k_lean26_batch");
-    return HP_OK;
+    if constexpr (WY == 32) {
+        if (blocks == 0) {  // either may be launched
+            const int rc = launch_lean_batch_nw<WY, FIELD, HASMP, 8>(d_args, d_start, R, 0, sweep_add, s);
+            if (rc) return rc;
+        } else if (lean_warps(blocks) == 8) {
+            return launch_lean_batch_nw<WY, FIELD, HASMP, 8>(d_args, d_start, R, blocks, sweep_add, s);
+        }
+    }
+    return launch_lean_batch_nw<WY, FIELD, HASMP, 4>(d_args, d_start, R, blocks, sweep_add, s);
 }
 
 template <int WY>
