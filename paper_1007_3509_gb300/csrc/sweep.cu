@@ -22,6 +22,7 @@
 // A site whose M neighbours all carry q_i cannot change; it skips the draw.
 #include <string.h>
 
+#include "routes.h"
 #include "sweep.cuh"
 
 namespace hp {
@@ -663,15 +664,14 @@ int plane_launch_batch(int nbr, int variant, int field, bool m, const PlaneArgs*
 // Variant a handle sweeps with until one is chosen (hp_set_sweep_variant or the
 // autotuner): the fastest measured on the benchmark lattices -- in 3D the lean
 // 64 x 32 window (512^3, grain field: 1.25e11 site-updates/s against 1.03e11 of
-// 64 x 44); in 2D the 128 x 28 lean tile (4 neighbours, 500^2 and 3000^2: 6.8 and
-// 33.0 us per MCS against 11.6 and 39.0 of 128 x 60; 8 neighbours, 1024^2: 11.2
-// against 14.8), but for 8 neighbours from 2048^2 sites on, where its halo costs
-// more than its latency saves, 128 x 60 (24.2 against 25.3; 3000^2: 40.3 against 46.4).
-int default_variant(const hp_handle* h) {
+// 64 x 44); in 2D the 128 x 28 or the 128 x 60 lean tile (tall_tiles; for the many
+// lattices of an ensemble, which fill the chip anyhow, 128 x 60 from 2^22 sites on, 8
+// neighbours).
+int default_variant(const hp_handle* h, bool one) {
+    const int64_t Lx = h->lat.L[0], Ly = h->lat.L[1];
     int v = 0;
     if (h->lat.nbr == 26) v = 11;
-    else if (h->lat.nbr == 4) v = 3;
-    else if (h->lat.nbr == 8) v = h->lat.N < (int64_t)1 << 22 ? 3 : 4;
+    else if (h->lat.dim == 2) v = tall_tiles(h->lat.nbr, Lx, Ly, h->mp || !one) ? 4 : 3;
     // variant 0 is built for every field mode; the others for the production ones
     return variant_ok(h->lat.nbr, v, h->desc.field_mode, h->mp != nullptr) ? v : 0;
 }
@@ -735,7 +735,7 @@ int sweep_run(hp_handle* h, int32_t n_mcs, cudaStream_t s) {
         return HP_OK;
     }
     const bool m = h->mp != nullptr;
-    const int v = h->an_J ? kAnisoVariant : h->sweep_variant >= 0 ? h->sweep_variant : default_variant(h);
+    const int v = h->an_J ? kAnisoVariant : h->sweep_variant >= 0 ? h->sweep_variant : default_variant(h, true);
     int32_t *qc = h->q, *mc = h->mp, *qa = h->q_alt, *ma = m ? h->mp_alt : nullptr;
     for (int32_t t = 0; t < n_mcs; ++t) {
         Range r_("mcs");
@@ -864,7 +864,7 @@ struct hp_ensemble {
 
 namespace {
 
-int ensemble_variant(const hp_ensemble* e) { return e->variant >= 0 ? e->variant : default_variant(e->m[0]); }
+int ensemble_variant(const hp_ensemble* e) { return e->variant >= 0 ? e->variant : default_variant(e->m[0], false); }
 
 int ensemble_build(hp_ensemble* e, cudaStream_t s) {
     const int variant = ensemble_variant(e);

@@ -1,0 +1,39 @@
+"""2D lattices on the route that their shape chooses (no kernel, no variant set), where the
+rules of csrc/routes.h change it.  Integer arithmetic: bit-exact against the oracle."""
+import numpy as np
+import pytest
+
+from paper_1007_3509_gb300 import synth
+from tests.gpu_util import need_gpu
+
+pytestmark = pytest.mark.gpu
+
+
+def _check(oracle, L, nbr, n, field=True, kT=0.9, sweep0=0, calls=1):
+    torch, hm = need_gpu()
+    G, seed = 12, 0xBEEF + nbr
+    q0 = synth.blocky_lattice(L, G, 4, block=9).astype(np.int32)
+    table = np.random.default_rng(7).integers(-200, 200, size=G).astype(np.int32) if field else None
+    lat = hm.Lattice(2, L, nbr, 256, seed, G, hm.FIELD_GRAIN if field else hm.FIELD_NONE)
+    q = torch.from_numpy(q0).cuda()
+    lat.hp_bind(q)
+    if field:
+        lat.hp_set_field(torch.from_numpy(table).cuda())
+    lat.hp_set_threshold_table(*hm.hp_build_threshold_table(kT))
+    lat.hp_set_sweep_counter(sweep0)
+    launches = hm.hp_kernel_launches()
+    for _ in range(calls):
+        lat.hp_sweep(n)
+    torch.cuda.synchronize()
+    launches = hm.hp_kernel_launches() - launches
+    assert hm.hp_sweep_status() == 0
+    thr, D = oracle.threshold_table(kT)
+    ref = oracle.sweep(2, L, nbr, 256, seed, sweep0, n * calls, thr, D, q0, table[q0] if field else None, None)[0]
+    np.testing.assert_array_equal(q.cpu().numpy(), ref)
+    lat.close()
+    return launches
+
+
+@pytest.mark.parametrize("L,nbr", [((1702, 1702), 8), ((1800, 1800), 8), ((1702, 1702), 4), ((1502, 1502), 8)])
+def test_tiles_short_and_tall(oracle, L, nbr):
+    _check(oracle, L, nbr, 2)

@@ -32,3 +32,16 @@ def test_few_windows_take_eight_warps(ask):
     large = [(126, 90, 78), (128, 128, 64), (128, 128, 128), (1024, 1024, 1024)]
     got = ask(*(f"lean_warps({_lean_windows(*L)})" for L in small + large))
     assert got == [8] * len(small) + [4] * len(large)
+
+
+def test_tall_tiles_where_short_ones_need_a_second_wave(ask):
+    """Lattices of 2.3 to 4.2 million sites that the short tiles swept slower."""
+    tall = [(8, 1362, 2300), (8, 1190, 3500), (8, 3002, 1000), (8, 1702, 1702), (8, 2046, 1500), (8, 1502, 2000),
+            (8, 1800, 1800), (8, 2044, 2044), (8, 2402, 1100), (8, 4096, 4096),
+            (4, 1702, 1702), (4, 3002, 1000), (4, 1502, 2000), (4, 1362, 2300), (4, 1922, 1960)]
+    short = [(8, 1502, 1502), (8, 1022, 2300), (8, 1202, 1202), (8, 3002, 700), (8, 500, 500),
+             (4, 1602, 1700), (4, 962, 2800), (4, 2046, 2046), (4, 2402, 2402), (4, 1800, 1800), (4, 2048, 2048), (4, 4096, 4096)]
+    got = ask(*(f"tall_tiles({n}, {x}, {y}, false)" for n, x, y in tall + short))
+    assert got == [1] * len(tall) + [0] * len(short)
+    # with material points, by sites alone
+    assert ask("tall_tiles(8, 1702, 1702, true)", "tall_tiles(8, 2048, 2048, true)", "tall_tiles(4, 3002, 3002, true)") == [0, 1, 0]
