@@ -29,6 +29,7 @@
 
 #include <atomic>
 
+#include "routes.h"
 #include "sweep.cuh"
 
 namespace hp {
@@ -54,11 +55,6 @@ struct ResBatch {
     int smem;      // dynamic shared memory of the launch, bytes
 };
 
-// Strips: row pairs are dealt out as evenly as they go, the first ones larger.
-__host__ __device__ inline int strip_rows(int Ly, int cs, int r) {
-    const int pairs = Ly / 2;
-    return 2 * (pairs / cs + (r < pairs % cs ? 1 : 0));
-}
 __host__ __device__ inline int strip_start(int Ly, int cs, int r) {
     const int pairs = Ly / 2, rem = pairs % cs;
     return 2 * (r * (pairs / cs) + (r < rem ? r : rem));
@@ -295,9 +291,7 @@ __global__ void __launch_bounds__(1024, 1) k_res2d(const __grid_constant__ ResBa
 }
 
 int warps_for(int nbr, int rows) {
-    const int lines = nbr == 8 ? rows / 2 : rows;  // rows worked at the same time
-    if (lines <= 32) return lines;
-    const int per = (lines + 31) / 32;
+    const int lines = strip_lines(nbr, rows), per = lines_per_warp(lines);
     return (lines + per - 1) / per;
 }
 
@@ -349,7 +343,7 @@ int res2d_cluster(hp_handle* const* m, int R) {
         const hp_handle* h = m[r];
         const int64_t Lx = h->lat.L[0], Ly = h->lat.L[1];
         if (h->lat.dim != 2 || h->mp || h->an_J || h->desc.field_mode == HP_FIELD_POINT || Lx > 2048 || Ly > 4096) return 0;
-        while (cs > 1 && Ly < 8 * cs) cs /= 2;  // at least eight rows a strip
+        cs = res_cluster(cs, Ly);
     }
     const int warps = res_warps(m, R, cs);
     for (int r = 0; r < R; ++r)

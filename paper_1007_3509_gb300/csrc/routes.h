@@ -42,4 +42,42 @@ inline bool tall_tiles(int nbr, int64_t Lx, int64_t Ly, bool hasmp) {
     return Lx % 4 != 0 && tiles_2d(Lx, Ly, 28) > 6 * kSMs && tiles_2d(Lx, Ly, 60) <= 4 * kSMs;
 }
 
+// ---- Resident 2D sweep (res2d.cu): one thread-block cluster per lattice ---------------
+// CTAs per cluster, from `cs` down: at least eight rows a strip.
+inline int res_cluster(int cs, int64_t Ly) {
+    while (cs > 1 && Ly < 8 * cs) cs /= 2;
+    return cs;
+}
+// Strips: row pairs are dealt out as evenly as they go, the first ones larger.
+HP_HD int strip_rows(int Ly, int cs, int r) {
+    const int pairs = Ly / 2;
+    return 2 * (pairs / cs + (r < pairs % cs ? 1 : 0));
+}
+// Lines of a strip that are worked at the same time (8 neighbours: row pairs), and the
+// lines each warp of at most 32 goes through.
+HP_HD int strip_lines(int nbr, int rows) { return nbr == 8 ? rows / 2 : rows; }
+inline int lines_per_warp(int lines) { return (lines + 31) / 32; }
+
+// Estimated us per MCS of one lattice on its cluster: the barriers, a chain per line of
+// a warp and pass over 128 columns, and the instructions of all passes.  Fitted to lattices of 50-site grains at kT = 1, 64^2 to 600^2
+// and 16 x 2000 to 2048 x 64: within 15 % (some coarse ones run 10 % below it).
+inline double res_us(int nbr, int64_t Lx, int64_t Ly, int cs) {
+    const int lines = strip_lines(nbr, strip_rows((int)Ly, cs, 0)), passes = (int)((Lx + 127) / 128);
+    const int chain = lines_per_warp(lines) * (1 + passes), work = lines * passes;
+    return nbr == 8 ? 1.0 + chain + 0.11 * work : 1.3 + 0.3 * chain + 0.07 * work;
+}
+
+// One lattice on its cluster?  Against the per-colour kernel's 3.7 us per MCS (4
+// neighbours, two launches) and 7.2 to 7.4 us (8 neighbours, four) on lattices of this
+// size: 4 neighbours by the passes of a strip, 8 neighbours by the estimate.  Per MCS on
+// the cluster / per colour: 4 neighbours 128^2 (16 passes) 2.9 / 3.7, 190 x 86 (24) 3.4 /
+// 3.6, 128 x 200 (26) 3.8 / 3.6, 120 x 240 4.3 / 3.6, 512 x 32 4.3 / 3.6, 2048 x 8 12.0 /
+// 3.6; 8 neighbours 256^2 6.8 / 7.3, 512 x 64 6.9 / 7.3, 128 x 500 7.3 / 7.3, 512 x 128
+// 7.9 / 7.4, 300 x 200 8.6 / 7.3, 64 x 1000 12.7 / 7.2, 2000 x 30 25.1 / 7.3, 16 x 4000
+// 33.1 / 7.2.
+inline bool one_resident(int nbr, int64_t Lx, int64_t Ly, int cs) {
+    if (nbr == 4) return strip_rows((int)Ly, cs, 0) * (int)((Lx + 127) / 128) <= 24;
+    return res_us(nbr, Lx, Ly, cs) <= 8.0;
+}
+
 }  // namespace hp

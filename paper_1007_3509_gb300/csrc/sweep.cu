@@ -676,29 +676,32 @@ int default_variant(const hp_handle* h, bool one) {
     return variant_ok(h->lat.nbr, v, h->desc.field_mode, h->mp != nullptr) ? v : 0;
 }
 
-// Cluster size when these lattices are better swept by the resident 2D kernel, else
-// 0.  One lattice, 8 neighbours: 8 SMs at 0.1 us per MCS and 1000 sites against the
-// tile kernel's floor of 7 to 8 us a launch (220^2: 6.7 us per MCS against 8.2; 250^2,
-// 6.7 against 11.1 without 16-byte rows; 300^2: 9.9 against 7.9).  4 neighbours: against
-// the per-colour kernel's 3.7 us per MCS (128^2, rows of one pass of a warp: 2.9;
-// 136^2: 4.3).  Several, whose launches cost 10 to 12 us: up to 300^2 each, or enough of
-// them to fill the chip (8 neighbours, kT = 1, 100 MCS: 32 x 500^2 6.0 ms against 6.7,
-// 100 x 500^2 14.0 against 19.5, but 4 x 500^2 2.0 against 1.6).
-int resident(hp_handle* const* m, int R) {
+// Cluster size when these lattices are better swept by the resident 2D kernel, else 0.
+// A handle's own sweep: one_resident.  Several, whose launches of tiles cost 10 to 12
+// us: up to 300^2 each, or enough of them to fill the chip (8 neighbours, kT = 1, 100
+// MCS: 32 x 500^2 6.0 ms against 6.7, 100 x 500^2 14.0 against 19.5, but 4 x 500^2 2.0
+// against 1.6).
+int resident(hp_handle* const* m, int R, bool ensemble) {
+    const int cs = res2d_cluster(m, R);
+    if (!cs) return 0;
+    const int nbr = m[0]->lat.nbr;
+    if (!ensemble) return one_resident(nbr, m[0]->lat.L[0], m[0]->lat.L[1], cs) ? cs : 0;
     int64_t sites = 0;
     for (int r = 0; r < R; ++r) sites += m[r]->lat.N;
-    const int cs = res2d_cluster(m, R);
-    const int64_t most = R > 1 ? 100000 : m[0]->lat.nbr == 4 ? 16384 : 65536;
-    return cs && (sites <= R * most || (int64_t)R * cs >= 152) ? cs : 0;
+    const int64_t most = R > 1 ? 100000 : nbr == 4 ? 16384 : 65536;
+    return sites <= R * most || (int64_t)R * cs >= kSMs ? cs : 0;
 }
 
-// Lattices that the per-colour kernel sweeps faster than the fused one: two chained
-// launches of one site a thread against a window's fill and halo.  us per MCS, 50 and
+// Lattices that the per-colour kernel sweeps faster than the fused one: chained launches
+// of one site a thread against a window's fill and halo.  4 neighbours, us per MCS, 50 and
 // 500 sites a grain: 256^2 3.8 and 3.8 against 8.4 and 6.8, 700^2 5.9 and 5.7 against 8.5
 // and 6.9, with material points 6.6 and 6.4 against 11.0 and 9.3; 1500^2 18.0 and 17.5
 // against 15.3 and 11.1.  With misorientation tables 300^2 9.4 and 7.5 against 13.0 and
-// 9.0, 360^2 11.5 and 10.0 against 13.0 and 9.0.
+// 9.0, 360^2 11.5 and 10.0 against 13.0 and 9.0.  8 neighbours, the small lattices
+// whose strips are too long for the cluster kernel: 2000 x 30 7.3 against 8.0, 64 x 1000
+// 7.2 against 12.4 (one_resident).
 bool per_colour(const hp_handle* h) {
+    if (h->lat.nbr == 8) return !h->an_J && !h->mp && h->lat.N <= 65536;
     return h->lat.nbr == 4 && h->lat.N < (h->an_J ? 100000 : (int64_t)1 << 19);
 }
 
@@ -716,7 +719,7 @@ int sweep_run(hp_handle* h, int32_t n_mcs, cudaStream_t s) {
                        (h->mp ? h->desc.field_mode == HP_FIELD_POINT : h->desc.field_mode != HP_FIELD_POINT);
     bool fused = nbr != 6 && (!h->an_J || tiles) && h->sweep_kernel != HP_SWEEP_PHASE;
     if (fused && h->sweep_kernel == HP_SWEEP_AUTO && h->sweep_variant < 0) {
-        const int cs = resident(&h, 1);
+        const int cs = resident(&h, 1, false);
         if (cs) {
             const int rc = res2d_run(&h, 1, cs, n_mcs, s);
             if (rc) return rc;
@@ -827,7 +830,7 @@ extern "C" int hp_sweep_autotune(hp_handle* h, int32_t n_mcs, float* ms_out, int
     h->sweep_kernel = kernel0;
     h->sweep_variant = best;
     // a lattice that the resident 2D kernel takes keeps to it when it beats them all
-    const int cs = rc == HP_OK && kernel0 == HP_SWEEP_AUTO ? resident(&h, 1) : 0;
+    const int cs = rc == HP_OK && kernel0 == HP_SWEEP_AUTO ? resident(&h, 1, false) : 0;
     if (cs && (rc = res2d_run(&h, 1, cs, 1, s)) == HP_OK) {
         cudaEventRecord(e0, s);
         rc = res2d_run(&h, 1, cs, n_mcs, s);
@@ -996,7 +999,7 @@ extern "C" int hp_ensemble_sweep(hp_ensemble* e, int32_t n_mcs, void* stream) {
     if (n_mcs == 0) return HP_OK;
     cudaStream_t s = as_stream(stream);
     int rc = HP_OK;
-    const int cs = e->variant < 0 ? resident(e->m.data(), (int)e->m.size()) : 0;
+    const int cs = e->variant < 0 ? resident(e->m.data(), (int)e->m.size(), true) : 0;
     if (cs) {
         if ((rc = res2d_run(e->m.data(), (int)e->m.size(), cs, n_mcs, s))) return rc;
         for (hp_handle* h : e->m) h->sweep += (uint64_t)n_mcs;
@@ -1079,7 +1082,7 @@ extern "C" int hp_ensemble_autotune(hp_ensemble* e, int32_t n_mcs, float* ms_out
     }
     e->variant = rc == HP_OK ? best : v0;
     // members that the resident 2D kernel takes keep to it when it beats every variant
-    const int R = (int)e->m.size(), cs = rc == HP_OK ? resident(e->m.data(), R) : 0;
+    const int R = (int)e->m.size(), cs = rc == HP_OK ? resident(e->m.data(), R, true) : 0;
     if (cs && (rc = res2d_run(e->m.data(), R, cs, 1, s)) == HP_OK) {
         cudaEventRecord(e0, s);
         rc = res2d_run(e->m.data(), R, cs, n_mcs, s);

@@ -37,3 +37,13 @@ def _check(oracle, L, nbr, n, field=True, kT=0.9, sweep0=0, calls=1):
 @pytest.mark.parametrize("L,nbr", [((1702, 1702), 8), ((1800, 1800), 8), ((1702, 1702), 4), ((1502, 1502), 8)])
 def test_tiles_short_and_tall(oracle, L, nbr):
     _check(oracle, L, nbr, 2)
+
+
+# launches of one call of n MCS: 1 on a cluster, n times the colours per colour
+@pytest.mark.parametrize("L,nbr,launches", [
+    ((128, 128), 4, 1), ((256, 64), 4, 1), ((120, 240), 4, 6), ((16, 1024), 4, 6), ((2048, 8), 4, 6), ((8, 2000), 4, 6),
+    ((256, 256), 8, 1), ((512, 64), 8, 1), ((64, 512), 8, 1), ((300, 200), 8, 12), ((2000, 30), 8, 12), ((2048, 16), 8, 12),
+    ((16, 4000), 8, 12), ((64, 1000), 8, 12)])
+@pytest.mark.parametrize("field", [False, True])
+def test_small_lattices_by_shape(oracle, L, nbr, launches, field):
+    assert _check(oracle, L, nbr, 3, field=field) == launches

@@ -45,3 +45,14 @@ def test_tall_tiles_where_short_ones_need_a_second_wave(ask):
     assert got == [1] * len(tall) + [0] * len(short)
     # with material points, by sites alone
     assert ask("tall_tiles(8, 1702, 1702, true)", "tall_tiles(8, 2048, 2048, true)", "tall_tiles(4, 3002, 3002, true)") == [0, 1, 0]
+
+
+def test_one_lattice_on_a_cluster_by_its_shape(ask):
+    """Long or wide strips that the cluster kernel swept slower than one launch per colour."""
+    cluster = [(4, 64, 64), (4, 128, 128), (4, 126, 130), (4, 256, 64), (4, 190, 86), (8, 64, 64), (8, 128, 128), (8, 128, 256),
+               (8, 256, 256), (8, 220, 220), (8, 512, 64), (8, 64, 512), (8, 120, 240)]
+    colour = [(4, 128, 200), (4, 120, 240), (4, 64, 256), (4, 512, 32), (4, 1024, 16), (4, 2048, 8), (4, 16, 1024), (4, 8, 2000),
+              (8, 512, 128), (8, 300, 200), (8, 180, 360), (8, 64, 1000), (8, 2000, 30), (8, 2048, 16), (8, 1022, 64),
+              (8, 16, 4000), (8, 32, 2000)]
+    got = ask(*(f"one_resident({n}, {x}, {y}, res_cluster(8, {y}))" for n, x, y in cluster + colour))
+    assert got == [1] * len(cluster) + [0] * len(colour)
