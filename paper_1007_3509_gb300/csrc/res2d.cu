@@ -315,24 +315,58 @@ size_t res_all(const hp_handle* h, int cs, int warps) {
     return all < (size_t)kSmemMax ? all : (size_t)kSmemMax;
 }
 
+// Launch of `members` clusters; at: room for its one attribute.
+template <int NBR, int FIELD>
+int config_res(int members, int cs, int warps, int smem, cudaStream_t s, cudaLaunchConfig_t* cfg, cudaLaunchAttribute* at) {
+    HP_CUDA(cudaFuncSetAttribute(k_res2d<NBR, FIELD>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax));
+    memset(cfg, 0, sizeof *cfg);
+    cfg->gridDim = dim3((unsigned)(members * cs));
+    cfg->blockDim = dim3((unsigned)(32 * warps));
+    cfg->dynamicSmemBytes = (size_t)smem;
+    cfg->stream = s;
+    at->id = cudaLaunchAttributeClusterDimension;
+    at->val.clusterDim.x = (unsigned)cs;
+    at->val.clusterDim.y = at->val.clusterDim.z = 1;
+    cfg->attrs = at;
+    cfg->numAttrs = cs > 1 ? 1 : 0;
+    return HP_OK;
+}
+
 template <int NBR, int FIELD>
 int launch_res(const ResBatch& b, int members, int warps, cudaStream_t s) {
-    HP_CUDA(cudaFuncSetAttribute(k_res2d<NBR, FIELD>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax));
     cudaLaunchConfig_t cfg;
-    memset(&cfg, 0, sizeof cfg);
-    cfg.gridDim = dim3((unsigned)(members * b.cs));
-    cfg.blockDim = dim3((unsigned)(32 * warps));
-    cfg.dynamicSmemBytes = (size_t)b.smem;
-    cfg.stream = s;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = (unsigned)b.cs;
-    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = b.cs > 1 ? 1 : 0;
+    cudaLaunchAttribute at;
+    const int rc = config_res<NBR, FIELD>(members, b.cs, warps, b.smem, s, &cfg, &at);
+    if (rc) return rc;
     count_launch();
     HP_CUDA(cudaLaunchKernelEx(&cfg, k_res2d<NBR, FIELD>, b));
     return HP_OK;
+}
+
+// Clusters of a launch that run at the same time (0: the query failed).
+template <int NBR, int FIELD>
+int active_res(int members, int cs, int warps, int smem) {
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute at;
+    int n = 0;
+    if (config_res<NBR, FIELD>(members, cs, warps, smem, nullptr, &cfg, &at)) return 0;
+    if (cs == 1) {
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_res2d<NBR, FIELD>, 32 * warps, (size_t)smem) != cudaSuccess) n = 0;
+        n *= kSMs;
+    } else if (cudaOccupancyMaxActiveClusters(&n, k_res2d<NBR, FIELD>, &cfg) != cudaSuccess) {
+        n = 0;
+    }
+    if (n <= 0) cudaGetLastError();
+    return n;
+}
+
+size_t res_smem(hp_handle* const* m, int R, int cs, int warps) {
+    size_t smem = 0;
+    for (int r = 0; r < R; ++r) {
+        const size_t want = res_all(m[r], cs, warps);
+        smem = want > smem ? want : smem;
+    }
+    return smem;
 }
 
 }  // namespace
@@ -351,6 +385,34 @@ int res2d_cluster(hp_handle* const* m, int R) {
     return cs;
 }
 
+// Estimated us per MCS of R lattices on clusters of cs, launch after launch: in each, the
+// members taken in order by the clusters that run at the same time.  -1: unknown.
+double res2d_us(hp_handle* const* m, int R, int cs) {
+    const int nbr = m[0]->lat.nbr, field = m[0]->desc.field_mode == HP_FIELD_GRAIN ? 1 : 0;
+    double total = 0.0;
+    for (int r0 = 0; r0 < R; r0 += kMembers) {
+        const int k = R - r0 < kMembers ? R - r0 : kMembers;
+        const int warps = res_warps(m + r0, k, cs), smem = (int)res_smem(m + r0, k, cs, warps);
+        int active = nbr == 8 ? (field ? active_res<8, 1>(k, cs, warps, smem) : active_res<8, 0>(k, cs, warps, smem))
+                              : (field ? active_res<4, 1>(k, cs, warps, smem) : active_res<4, 0>(k, cs, warps, smem));
+        if (active < 1) return -1.0;
+        const int per_sm = active * cs < kSMs ? 1 : (active * cs + kSMs / 2) / kSMs;  // CTAs an SM takes
+        if (active > k) active = k;
+        double busy[kMembers] = {}, most = 0.0;
+        for (int i = 0; i < k; ++i) {
+            int at = 0;
+            for (int c = 1; c < active; ++c)
+                if (busy[c] < busy[at]) at = c;
+            const int first = i / active * active, wave = k - first < active ? k - first : active;
+            const int asked = (wave * cs + kSMs - 1) / kSMs;  // CTAs an SM has in this member's wave
+            busy[at] += res_us(nbr, m[r0 + i]->lat.L[0], m[r0 + i]->lat.L[1], cs, asked < per_sm ? asked : per_sm);
+            most = busy[at] > most ? busy[at] : most;
+        }
+        total += most;
+    }
+    return total;
+}
+
 int res2d_run(hp_handle* const* m, int R, int cs, int32_t n_mcs, cudaStream_t s) {
     const int nbr = m[0]->lat.nbr, field = m[0]->desc.field_mode == HP_FIELD_GRAIN ? 1 : 0;
     for (int32_t done = 0; done < n_mcs; done += kMcsPerLaunch) {
@@ -362,7 +424,6 @@ int res2d_run(hp_handle* const* m, int R, int cs, int32_t n_mcs, cudaStream_t s)
             b.cs = cs;
             b.n_mcs = n;
             const int warps = res_warps(m + r0, k, cs);
-            size_t smem = 0;
             for (int i = 0; i < k; ++i) {
                 const hp_handle* h = m[r0 + i];
                 ResArgs& a = b.m[i];
@@ -376,10 +437,8 @@ int res2d_run(hp_handle* const* m, int R, int cs, int32_t n_mcs, cudaStream_t s)
                 a.J = h->desc.J_fix;
                 a.Lx = (int)h->lat.L[0];
                 a.Ly = (int)h->lat.L[1];
-                const size_t want = res_all(h, cs, warps);
-                smem = want > smem ? want : smem;
             }
-            b.smem = (int)smem;
+            b.smem = (int)res_smem(m + r0, k, cs, warps);
             const int rc = nbr == 8 ? (field ? launch_res<8, 1>(b, k, warps, s) : launch_res<8, 0>(b, k, warps, s))
                                     : (field ? launch_res<4, 1>(b, k, warps, s) : launch_res<4, 0>(b, k, warps, s));
             if (rc) return rc;

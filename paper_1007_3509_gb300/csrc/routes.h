@@ -58,12 +58,13 @@ HP_HD int strip_rows(int Ly, int cs, int r) {
 HP_HD int strip_lines(int nbr, int rows) { return nbr == 8 ? rows / 2 : rows; }
 inline int lines_per_warp(int lines) { return (lines + 31) / 32; }
 
-// Estimated us per MCS of one lattice on its cluster: the barriers, a chain per line of
-// a warp and pass over 128 columns, and the instructions of all passes.  Fitted to lattices of 50-site grains at kT = 1, 64^2 to 600^2
+// Estimated us per MCS of one lattice on its cluster, `sharing` CTAs to an SM: the
+// barriers, a chain per line of a warp and pass over 128 columns, and the instructions
+// of all passes of the SM.  Fitted to lattices of 50-site grains at kT = 1, 64^2 to 600^2
 // and 16 x 2000 to 2048 x 64: within 15 % (some coarse ones run 10 % below it).
-inline double res_us(int nbr, int64_t Lx, int64_t Ly, int cs) {
+inline double res_us(int nbr, int64_t Lx, int64_t Ly, int cs, int sharing = 1) {
     const int lines = strip_lines(nbr, strip_rows((int)Ly, cs, 0)), passes = (int)((Lx + 127) / 128);
-    const int chain = lines_per_warp(lines) * (1 + passes), work = lines * passes;
+    const int chain = lines_per_warp(lines) * (1 + passes), work = lines * passes * sharing;
     return nbr == 8 ? 1.0 + chain + 0.11 * work : 1.3 + 0.3 * chain + 0.07 * work;
 }
 
@@ -79,5 +80,24 @@ inline bool one_resident(int nbr, int64_t Lx, int64_t Ly, int cs) {
     if (nbr == 4) return strip_rows((int)Ly, cs, 0) * (int)((Lx + 127) / 128) <= 24;
     return res_us(nbr, Lx, Ly, cs) <= 8.0;
 }
+
+// An ensemble's launches of short tiles, us per MCS: a floor (longer where a window is
+// wider than a lattice) and so much per tile, a fifth more where a window is not fetched
+// by bulk copies.  `built`: the field mode has these tiles; the plane kernel otherwise.
+struct TileCost {
+    double tiles = 0.0;
+    bool narrow = false;
+    void add(int64_t Lx, int64_t Ly) {
+        const bool slow = Lx % 4 != 0 || Lx < 128 || Ly < 32;
+        tiles += (double)tiles_2d(Lx, Ly, 28) * (slow ? 1.2 : 1.0);
+        narrow = narrow || Lx < 128;
+    }
+    double us(int nbr, bool built) const {
+        const double floor = (built ? (nbr == 8 ? 12.0 : 11.2) : (nbr == 8 ? 24.0 : 22.0)) * (narrow ? 1.4 : 1.0);
+        const double t = built ? (nbr == 8 ? 6.0 + 0.024 * tiles : 5.0 + 0.0192 * tiles)
+                               : (nbr == 8 ? 15.0 + 0.029 * tiles : 12.0 + 0.026 * tiles);
+        return t > floor ? t : floor;
+    }
+};
 
 }  // namespace hp

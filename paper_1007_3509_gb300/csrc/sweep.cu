@@ -677,19 +677,27 @@ int default_variant(const hp_handle* h, bool one) {
 }
 
 // Cluster size when these lattices are better swept by the resident 2D kernel, else 0.
-// A handle's own sweep: one_resident.  Several, whose launches of tiles cost 10 to 12
-// us: up to 300^2 each, or enough of them to fill the chip (8 neighbours, kT = 1, 100
-// MCS: 32 x 500^2 6.0 ms against 6.7, 100 x 500^2 14.0 against 19.5, but 4 x 500^2 2.0
-// against 1.6).
+// A handle's own sweep: one_resident.  An ensemble, of members of up to some 300^2 or
+// clusters enough to fill the chip, by the estimates of both (res2d_us, TileCost): its
+// launches of tiles are not chained, and on the other side the longest member or the
+// last wave of clusters counts.  8 neighbours, 50-site grains at kT = 1, us per MCS
+// resident / tiles: 32 x 500^2 61 / 75, 16 x 500^2 41 / 40, 4 x 500^2 21 / 16, 24 x 300^2
+// 22 / 29, 32 x (2048 x 64) 83 / 48, one 600^2 with seven 64^2 33 / 18, one 400 x 1000
+// with fifteen 64^2 39 / 19.
 int resident(hp_handle* const* m, int R, bool ensemble) {
     const int cs = res2d_cluster(m, R);
     if (!cs) return 0;
     const int nbr = m[0]->lat.nbr;
     if (!ensemble) return one_resident(nbr, m[0]->lat.L[0], m[0]->lat.L[1], cs) ? cs : 0;
+    TileCost tiles;
     int64_t sites = 0;
-    for (int r = 0; r < R; ++r) sites += m[r]->lat.N;
-    const int64_t most = R > 1 ? 100000 : nbr == 4 ? 16384 : 65536;
-    return sites <= R * most || (int64_t)R * cs >= kSMs ? cs : 0;
+    for (int r = 0; r < R; ++r) {
+        tiles.add(m[r]->lat.L[0], m[r]->lat.L[1]);
+        sites += m[r]->lat.N;
+    }
+    if (sites > (int64_t)R * 100000 && R * cs < kSMs) return 0;
+    const double us = res2d_us(m, R, cs);
+    return us >= 0.0 && us <= 1.07 * tiles.us(nbr, m[0]->desc.field_mode == HP_FIELD_GRAIN) ? cs : 0;
 }
 
 // Lattices that the per-colour kernel sweeps faster than the fused one: chained launches

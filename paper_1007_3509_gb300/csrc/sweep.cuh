@@ -277,6 +277,8 @@ int lean_status(int* timed_out);
 // Resident 2D sweep (res2d.cu): cluster size for these lattices (all of one dim, nbr,
 // field mode), 0 when one of them does not fit or is of another kind.
 int res2d_cluster(hp_handle* const* m, int R);
+// Estimated us per MCS of an ensemble there, -1 when unknown.
+double res2d_us(hp_handle* const* m, int R, int cs);
 // n_mcs MCS of every lattice, in place, from each handle's sweep counter (not
 // advanced here).
 int res2d_run(hp_handle* const* m, int R, int cs, int32_t n_mcs, cudaStream_t s);

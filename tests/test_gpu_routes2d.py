@@ -47,3 +47,35 @@ def test_tiles_short_and_tall(oracle, L, nbr):
 @pytest.mark.parametrize("field", [False, True])
 def test_small_lattices_by_shape(oracle, L, nbr, launches, field):
     assert _check(oracle, L, nbr, 3, field=field) == launches
+
+
+# members, launches of one call of 3 MCS: 1 on clusters, 3 of tiles
+@pytest.mark.parametrize("shapes,launches", [
+    ([(64, 64)] * 5, 1), ([(400, 1000)] + [(64, 64)] * 15, 3), ([(600, 600)] + [(64, 64)] * 7, 3),
+    ([(500, 500)] * 24, 1), ([(128, 130), (300, 66), (64, 512)] * 4, 1), ([(72, 64)], 1)])
+@pytest.mark.parametrize("nbr", [4, 8])
+def test_ensembles_by_shape(oracle, shapes, launches, nbr):
+    torch, hm = need_gpu()
+    G, n, members = 12, 3, []
+    table = np.random.default_rng(7).integers(-200, 200, size=G).astype(np.int32)
+    for r, L in enumerate(shapes):
+        q0 = synth.blocky_lattice(L, G, r, block=9).astype(np.int32)
+        lat = hm.Lattice(2, L, nbr, 256, 40 + r, G, hm.FIELD_GRAIN)
+        q = torch.from_numpy(q0).cuda()
+        lat.hp_bind(q)
+        lat.hp_set_field(torch.from_numpy(table).cuda())
+        lat.hp_set_threshold_table(*hm.hp_build_threshold_table(0.5 + 0.02 * r))
+        members.append((lat, q, q0, L, 40 + r, 0.5 + 0.02 * r))
+    ens = hm.Ensemble([m[0] for m in members])
+    ens.hp_ensemble_sweep(n)
+    before = hm.hp_kernel_launches()
+    ens.hp_ensemble_sweep(n)
+    torch.cuda.synchronize()
+    assert hm.hp_kernel_launches() - before == launches
+    for lat, q, q0, L, seed, kT in members:
+        thr, D = oracle.threshold_table(kT)
+        ref = oracle.sweep(2, L, nbr, 256, seed, 0, 2 * n, thr, D, q0, table[q0], None)[0]
+        np.testing.assert_array_equal(q.cpu().numpy(), ref)
+    ens.close()
+    for m in members:
+        m[0].close()

@@ -56,3 +56,20 @@ def test_one_lattice_on_a_cluster_by_its_shape(ask):
               (8, 16, 4000), (8, 32, 2000)]
     got = ask(*(f"one_resident({n}, {x}, {y}, res_cluster(8, {y}))" for n, x, y in cluster + colour))
     assert got == [1] * len(cluster) + [0] * len(colour)
+
+
+def _ensemble_us(ask, nbr, shapes, sharing=1):
+    tiles = "[] { TileCost t; " + "".join(f"t.add({x}, {y}); " for x, y in shapes) + f"return t.us({nbr}, true); }}()"
+    return ask(tiles, *(f"res_us({nbr}, {x}, {y}, 8, {sharing})" for x, y in shapes))
+
+
+def test_ensembles_estimate_the_longest_member_and_the_tiles(ask):
+    """Measured us per MCS (50-site grains, kT = 1) of one wave of clusters and of the tiles."""
+    for nbr, shapes, cluster, tiles in [
+            (8, [(600, 600)] + [(64, 64)] * 7, 33.0, 17.7), (8, [(400, 1000)] + [(64, 64)] * 14, 38.9, 18.6),
+            (8, [(2048, 64)] * 8, 28.1, 16.2), (8, [(500, 500)] * 8, 20.7, 22.7), (8, [(300, 300)] * 8, 11.1, 14.2),
+            (8, [(200, 200)] * 8, 7.0, 12.4), (8, [(64, 1000)] * 8, 13.4, 19.9), (4, [(600, 600)] * 8, 30.0, 23.8),
+            (4, [(256, 256)] * 8, 6.8, 11.4), (4, [(2048, 64)] * 8, 16.0, 12.6), (4, [(400, 1000)] + [(64, 64)] * 14, 37.0, 15.7)]:
+        t, *m = _ensemble_us(ask, nbr, shapes)
+        assert abs(max(m) / cluster - 1) < 0.2 and abs(t / tiles - 1) < 0.3, (nbr, shapes[0], t, max(m))
+        assert (max(m) <= 1.07 * t) == (cluster <= tiles), (nbr, shapes[0], t, max(m))
