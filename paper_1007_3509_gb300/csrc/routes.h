@@ -42,6 +42,25 @@ inline bool tall_tiles(int nbr, int64_t Lx, int64_t Ly, bool hasmp) {
     return Lx % 4 != 0 && tiles_2d(Lx, Ly, 28) > 6 * kSMs && tiles_2d(Lx, Ly, 60) <= 4 * kSMs;
 }
 
+// 2D lattices that the per-colour kernel sweeps faster than the tiles: chained launches of
+// one site a thread against a window's fill and halo.  us per MCS, per colour / tiles, 50
+// and 500 sites a grain:
+//  * 4 neighbours, two launches: 256^2 3.8 and 3.8 / 8.4 and 6.8, 700^2 5.9 and 5.7 / 8.5
+//    and 6.9, with material points 6.6 and 6.4 / 11.0 and 9.3, 1500^2 18.0 and 17.5 / 15.3
+//    and 11.1; with misorientation tables 300^2 9.4 and 7.5 / 13.0 and 9.0, 360^2 11.5 and
+//    10.0 / 13.0 and 9.0;
+//  * 8 neighbours, four launches: lattices that the cluster kernel would take but for
+//    their long strips (one_resident): 2000 x 30 7.3 / 8.0, 64 x 1000 7.2 / 12.4;
+//  * lattices narrower than a window of 128 columns, which goes through theirs twice and
+//    more: 4 neighbours 16 x 60000 7.1 / 33.1, 126 x 8000 9.2 / 14.7, with tables 16 x 8000
+//    8.9 and 6.7 / 21.8 and 15.9, 100 x 4000 12.1 and 11.2 / 17.9 and 13.2; 8 neighbours up
+//    to 64 columns, 16 x 60000 11.4 / 38.6, 64 x 20000 15.3 / 21.0, with tables 16 x 60000
+//    36.5 and 24.6 / 181 and 90, but 100 x 4000 32.3 and 23.0 / 31.2 and 19.4.
+inline bool per_colour_2d(int nbr, int64_t Lx, int64_t N, bool tables, bool hasmp) {
+    if (nbr == 4) return Lx < 128 || N < (tables ? 100000 : (int64_t)1 << 19);
+    return Lx <= 64 || (!tables && !hasmp && N <= 65536);
+}
+
 // ---- Resident 2D sweep (res2d.cu): one thread-block cluster per lattice ---------------
 // CTAs per cluster, from `cs` down: at least eight rows a strip.
 inline int res_cluster(int cs, int64_t Ly) {

@@ -700,17 +700,8 @@ int resident(hp_handle* const* m, int R, bool ensemble) {
     return us >= 0.0 && us <= 1.07 * tiles.us(nbr, m[0]->desc.field_mode == HP_FIELD_GRAIN) ? cs : 0;
 }
 
-// Lattices that the per-colour kernel sweeps faster than the fused one: chained launches
-// of one site a thread against a window's fill and halo.  4 neighbours, us per MCS, 50 and
-// 500 sites a grain: 256^2 3.8 and 3.8 against 8.4 and 6.8, 700^2 5.9 and 5.7 against 8.5
-// and 6.9, with material points 6.6 and 6.4 against 11.0 and 9.3; 1500^2 18.0 and 17.5
-// against 15.3 and 11.1.  With misorientation tables 300^2 9.4 and 7.5 against 13.0 and
-// 9.0, 360^2 11.5 and 10.0 against 13.0 and 9.0.  8 neighbours, the small lattices
-// whose strips are too long for the cluster kernel: 2000 x 30 7.3 against 8.0, 64 x 1000
-// 7.2 against 12.4 (one_resident).
 bool per_colour(const hp_handle* h) {
-    if (h->lat.nbr == 8) return !h->an_J && !h->mp && h->lat.N <= 65536;
-    return h->lat.nbr == 4 && h->lat.N < (h->an_J ? 100000 : (int64_t)1 << 19);
+    return h->lat.dim == 2 && per_colour_2d(h->lat.nbr, h->lat.L[0], h->lat.N, h->an_J != nullptr, h->mp != nullptr);
 }
 
 int sweep_variants(int nbr) { return n_variants(nbr); }

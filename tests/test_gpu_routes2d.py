@@ -79,3 +79,38 @@ def test_ensembles_by_shape(oracle, shapes, launches, nbr):
     ens.close()
     for m in members:
         m[0].close()
+
+
+@pytest.mark.parametrize("L", [(2, 40000), (16, 9000), (64, 2000), (66, 2000), (126, 900)])
+@pytest.mark.parametrize("nbr", [4, 8])
+@pytest.mark.parametrize("mode", ["none", "grain", "point"])
+@pytest.mark.parametrize("tables", [False, True])
+def test_narrow_lattices(oracle, L, nbr, mode, tables):
+    torch, hm = need_gpu()
+    G, n, kT, N = 9, 3, 0.9, L[0] * L[1]
+    rng = np.random.default_rng(N)
+    q0 = synth.blocky_lattice(L, G, 31, block=3).astype(np.int32)
+    ang = rng.integers(0, 90000, size=G).astype(np.int32)
+    mp0 = rng.integers(0, N, size=N).astype(np.int32) if mode == "point" else None
+    table = None if mode == "none" else rng.integers(-40, 40, size=N if mode == "point" else G).astype(np.int32)
+    lat = hm.Lattice(2, L, nbr, 256, 0xA11, G, {"none": hm.FIELD_NONE, "grain": hm.FIELD_GRAIN, "point": hm.FIELD_POINT}[mode])
+    q, m = torch.from_numpy(q0).cuda(), None if mp0 is None else torch.from_numpy(mp0).cuda()
+    lat.hp_bind(q, m)
+    if table is not None:
+        lat.hp_set_field(torch.from_numpy(table).cuda())
+    lat.hp_set_threshold_table(*hm.hp_build_threshold_table(kT))
+    thr, D = oracle.threshold_table(kT)
+    b = None if table is None else table[q0 if mode == "grain" else mp0]
+    if tables:
+        J, mob = hm.hp_build_read_shockley(1.0, 15.0, 500, 91, 1000, mobility=True)
+        ta = torch.from_numpy(ang).cuda()
+        lat.hp_set_anisotropy(ta, 90000, 500, J, mob)
+        rq, _, rm, _ = oracle.sweep_aniso(2, L, nbr, 0xA11, 0, n, thr, D, q0, ang, 90000, 500, J, mob, b, mp0)
+    else:
+        rq, _, rm, _ = oracle.sweep(2, L, nbr, 256, 0xA11, 0, n, thr, D, q0, b, mp0)
+    lat.hp_sweep(n)
+    torch.cuda.synchronize()
+    np.testing.assert_array_equal(q.cpu().numpy(), rq)
+    if mp0 is not None:
+        np.testing.assert_array_equal(m.cpu().numpy(), rm)
+    lat.close()

@@ -73,3 +73,14 @@ def test_ensembles_estimate_the_longest_member_and_the_tiles(ask):
         t, *m = _ensemble_us(ask, nbr, shapes)
         assert abs(max(m) / cluster - 1) < 0.2 and abs(t / tiles - 1) < 0.3, (nbr, shapes[0], t, max(m))
         assert (max(m) <= 1.07 * t) == (cluster <= tiles), (nbr, shapes[0], t, max(m))
+
+
+def test_narrow_lattices_go_per_colour(ask):
+    """Lattices that a window of 128 columns goes through several times over."""
+    def rule(n, x, y, tables=0, mp=0):
+        return f"per_colour_2d({n}, {x}, {x * y}LL, {tables}, {mp})"
+    colour = [rule(4, 16, 8000, 1), rule(4, 16, 60000, 1), rule(4, 100, 4000, 1), rule(4, 16, 60000), rule(4, 126, 8000, 0, 1),
+              rule(8, 16, 60000), rule(8, 16, 60000, 1), rule(8, 64, 20000, 0, 1), rule(4, 700, 700), rule(8, 2000, 30)]
+    tiles = [rule(4, 128, 2000, 1), rule(4, 360, 360, 1), rule(4, 1024, 1024), rule(8, 100, 4000, 1), rule(8, 128, 600),
+             rule(8, 128, 128, 0, 1), rule(8, 256, 256, 1)]
+    assert ask(*colour, *tiles) == [1] * len(colour) + [0] * len(tiles)
