@@ -58,7 +58,7 @@ extern "C" {
                           /* HP_ORIENT_ANGLE angle t about z (Sec. 5), float[4G]     */
 
 /* Sweep kernel choice (hp_set_sweep_kernel). */
-#define HP_SWEEP_AUTO 0   /* the route measured fastest for the lattice       */
+#define HP_SWEEP_AUTO 0   /* chosen by the lattice's size, shape and field    */
 #define HP_SWEEP_PHASE 1  /* one launch per colour phase, in place              */
 #define HP_SWEEP_FUSED 2  /* all phases of a plane in shared memory, double-buffered */
 
@@ -243,15 +243,20 @@ HP_API int hp_sweep(hp_handle* h, int32_t n_mcs, void* stream);
  * 26-neighbour lattice, lean 3D windows (64 x 44, 40, 36, 32: variants 8-11;
  * every random number drawn while the window is in flight).  Until a variant is
  * chosen, a handle sweeps with the fastest measured for its kind of lattice:
- * variant 11 in 3D, 3 or 4 in 2D; a small 2D lattice without material points is
- * instead kept in the shared memory of a thread-block cluster for the whole call.
+ * variant 11 in 3D, 3 or 4 in 2D, where these are built for its field mode, else 0.
+ * Some 2D lattices are swept by another kernel until then: small ones without
+ * material points are kept in the shared memory of a thread-block cluster for the
+ * whole call, 4-neighbour ones of up to 2^19 sites, narrow ones and small ones with
+ * long rows go per colour.
  * hp_sweep_variants: how many exist for `nbr`.
  * hp_set_sweep_variant: choose one (HP_ERR_ARG if not built for the handle's
  * field mode).  hp_sweep_autotune: time every variant for n_mcs MCS on a
  * backup of the bound state (the lattice and sweep counter are restored),
- * keep the fastest (or the resident 2D kernel, where the lattice takes it and it
- * beats them all), write per-variant milliseconds to ms_out (host float[n], -1
- * for unavailable variants; may be NULL) and the fastest variant to *chosen.
+ * keep the fastest, write per-variant milliseconds to ms_out (host float[n], -1
+ * for unavailable variants; may be NULL) and the fastest variant to *chosen.  A
+ * lattice whose own route is another kernel keeps to that, whatever *chosen is, when
+ * it beats them all; with misorientation tables set no variant has a part in the
+ * sweep and the handle's choice stays as it was.
  * Allocates a temporary copy of the lattice; synchronises `stream`.          */
 HP_API int hp_sweep_variants(int32_t nbr, int32_t* n);
 HP_API int hp_set_sweep_variant(hp_handle* h, int32_t v);

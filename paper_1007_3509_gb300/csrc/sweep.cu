@@ -717,7 +717,8 @@ int sweep_run(hp_handle* h, int32_t n_mcs, cudaStream_t s) {
     const bool tiles = h->an_J && h->lat.dim == 2 &&
                        (h->mp ? h->desc.field_mode == HP_FIELD_POINT : h->desc.field_mode != HP_FIELD_POINT);
     bool fused = nbr != 6 && (!h->an_J || tiles) && h->sweep_kernel != HP_SWEEP_PHASE;
-    if (fused && h->sweep_kernel == HP_SWEEP_AUTO && h->sweep_variant < 0) {
+    // (which have one shape there: a chosen variant says nothing about them)
+    if (fused && h->sweep_kernel == HP_SWEEP_AUTO && (h->sweep_variant < 0 || h->an_J)) {
         const int cs = resident(&h, 1, false);
         if (cs) {
             const int rc = res2d_run(&h, 1, cs, n_mcs, s);
@@ -796,7 +797,12 @@ extern "C" int hp_sweep_autotune(hp_handle* h, int32_t n_mcs, float* ms_out, int
     cudaMemcpyAsync(bq, h->q, bytes, cudaMemcpyDeviceToDevice, s);
     if (m) cudaMemcpyAsync(bm, h->mp, bytes, cudaMemcpyDeviceToDevice, s);
     const uint64_t sweep0 = h->sweep;
-    const int kernel0 = h->sweep_kernel;
+    const int kernel0 = h->sweep_kernel, variant0 = h->sweep_variant;
+    auto restore = [&]() {
+        cudaMemcpyAsync(h->q, bq, bytes, cudaMemcpyDeviceToDevice, s);
+        if (m) cudaMemcpyAsync(h->mp, bm, bytes, cudaMemcpyDeviceToDevice, s);
+        h->sweep = sweep0;
+    };
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
@@ -810,9 +816,7 @@ extern "C" int hp_sweep_autotune(hp_handle* h, int32_t n_mcs, float* ms_out, int
         h->sweep = sweep0;
         rc = sweep_run(h, 1, s);  // warm-up (also configures the kernel)
         if (rc) break;
-        cudaMemcpyAsync(h->q, bq, bytes, cudaMemcpyDeviceToDevice, s);
-        if (m) cudaMemcpyAsync(h->mp, bm, bytes, cudaMemcpyDeviceToDevice, s);
-        h->sweep = sweep0;
+        restore();
         cudaEventRecord(e0, s);
         rc = sweep_run(h, n_mcs, s);
         cudaEventRecord(e1, s);
@@ -822,23 +826,26 @@ extern "C" int hp_sweep_autotune(hp_handle* h, int32_t n_mcs, float* ms_out, int
         cudaEventElapsedTime(&ms, e0, e1);
         if (ms_out) ms_out[v] = ms;
         if (ms < best_ms) { best_ms = ms; best = v; }
-        cudaMemcpyAsync(h->q, bq, bytes, cudaMemcpyDeviceToDevice, s);
-        if (m) cudaMemcpyAsync(h->mp, bm, bytes, cudaMemcpyDeviceToDevice, s);
+        restore();
     }
     h->sweep = sweep0;
     h->sweep_kernel = kernel0;
     h->sweep_variant = best;
-    // a lattice that the resident 2D kernel takes keeps to it when it beats them all
-    const int cs = rc == HP_OK && kernel0 == HP_SWEEP_AUTO ? resident(&h, 1, false) : 0;
-    if (cs && (rc = res2d_run(&h, 1, cs, 1, s)) == HP_OK) {
+    if (rc == HP_OK && h->an_J) {
+        h->sweep_variant = variant0;  // no variant has a part in it: all were the same sweep
+    } else if (rc == HP_OK && kernel0 == HP_SWEEP_AUTO && (resident(&h, 1, false) || per_colour(h))) {
+        // a lattice whose own route is none of the variants keeps to it when it beats them all
+        h->sweep_variant = -1;
+        rc = sweep_run(h, 1, s);  // warm-up
+        restore();
         cudaEventRecord(e0, s);
-        rc = res2d_run(&h, 1, cs, n_mcs, s);
+        if (rc == HP_OK) rc = sweep_run(h, n_mcs, s);
         cudaEventRecord(e1, s);
         float ms = 0.0f;
-        if (rc == HP_OK && cudaEventSynchronize(e1) == cudaSuccess && cudaEventElapsedTime(&ms, e0, e1) == cudaSuccess &&
-            ms < best_ms)
-            h->sweep_variant = -1;
-        cudaMemcpyAsync(h->q, bq, bytes, cudaMemcpyDeviceToDevice, s);
+        if (rc != HP_OK || cudaEventSynchronize(e1) != cudaSuccess || cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess ||
+            ms >= best_ms)
+            h->sweep_variant = best;
+        restore();
     }
     cudaFreeAsync(bq, s);
     if (bm) cudaFreeAsync(bm, s);
