@@ -157,8 +157,9 @@ __device__ __noinline__ double newton_slip(double at, double k, double taus, dou
 // x^2 (c2 - c3 x) / K is at most q y / 2 of x and each fixed-point step shrinks
 // its error by a factor q y, so three steps in FP32 leave it below 1e-10.  Other
 // slips take Newton on the exact FP64 residual, and so that the committed FP32 slip
-// and resistance are those of FP64 arithmetic throughout, a result within 2^-14 of
-// halfway between two FP32 numbers is formed again in FP64 (one in 8000).
+// and resistance are those of FP64 arithmetic throughout, with and without hardening, a
+// result within 2^-14 of halfway between two FP32 numbers is formed again in FP64 (one
+// in 8000).
 __device__ __forceinline__ Pair two_sum(float a, float b) {
     const float s = __fadd_rn(a, b), t = __fsub_rn(s, a);
     return Pair{s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t))};
@@ -168,16 +169,22 @@ __device__ __forceinline__ Pair fast_sum(float a, float b) {  // |a| >= |b|
     return Pair{s, __fsub_rn(b, __fsub_rn(s, a))};
 }
 
-// |lo| within 2^-14 of half a unit in the last place of hi: rounding the sum to
-// FP32 may go either way with an error of 2^-46
+// v > 0 within 2^-14 of halfway between two FP32 numbers: rounding the sum to FP32 may go
+// either way with an error of 2^-46.  Below a power of two the numbers lie half as far
+// apart as above it.
 __device__ __forceinline__ bool near_half(Pair v) {
-    const float half = __int_as_float((__float_as_int(v.hi) & 0x7F800000) - (24 << 23));
+    const int below = (int)((uint32_t)__float_as_int(v.lo) >> 31);
+    const float half = __int_as_float(((__float_as_int(v.hi) - below) & 0x7F800000) - (24 << 23));
     return fabsf(v.lo) > half * (1.0f - 0x1p-14f);
 }
-// The map in FP64: the series where its bound holds, Newton otherwise.  Not inlined
-// (rare; see newton_slip).
+// The map in FP64: the quotient without hardening; with it the series where its bound
+// holds, Newton otherwise.  Not inlined (rare; see newton_slip).
 __device__ __noinline__ Pair slip_fp64(float at_f, float g, double k, const RMConsts& c, float* g_new) {
     const double at = at_f, sat = c.taus - (double)g, K = k + sat * c.hr;
+    if (!c.hard) {
+        *g_new = g;
+        return pair_of((at - (double)g) / k);
+    }
     const float rKf = 1.0f / (float)K;
     double rK = (double)rKf;
     rK = rK * (2.0 - K * rK);
@@ -215,7 +222,7 @@ __device__ __forceinline__ Pair return_map(float at, float g, Pair k, double kd,
     Pair x = fast_sum(q0, __fmul_rn(rem, rK));
     if (!c.hard) {
         *g_new = g;
-        return x;
+        return near_half(x) ? slip_fp64(at, g, kd, c, g_new) : x;
     }
     const float sr = (c.taus32 - g) * rK;  // sat / K
     const float y = c.hr32 * x.hi, q = c.hr32 * sr;
