@@ -414,7 +414,7 @@ __global__ void __launch_bounds__(LeanCfg<WY, FIELD, HASMP, NW>::kLT, LeanCfg<WY
 
 // Many independent lattices in one launch: block b belongs to the replica r
 // with start[r] <= b < start[r+1]; within it b - start[r] = zidx * tiles + tile.
-// Windows are filled by the asynchronous 16-byte copies.
+// Windows are filled by the asynchronous copies, 16 or 8 bytes, or by single loads.
 template <int WY, int FIELD, bool HASMP, int NW>
 __global__ void __launch_bounds__(LeanCfg<WY, FIELD, HASMP, NW>::kLT, LeanCfg<WY, FIELD, HASMP, NW>::MINB)
     k_lean26_batch(const PlaneArgs* __restrict__ args, const int64_t* __restrict__ start, int R, uint32_t sweep_add) {
@@ -455,7 +455,7 @@ PFN_cuTensorMapEncodeTiled_v12000 map_encoder() {
 
 // Descriptor of one int32 lattice array (Lx x Ly x Lz) with a 64 x WY x 1 box;
 // false when it cannot be encoded (the kernel then copies every window with
-// asynchronous 16-byte copies instead).
+// asynchronous copies, or single loads, instead).
 bool encode_box(CUtensorMap* m, const void* base, const PlaneArgs& a, int WY) {
     memset(m, 0, sizeof(*m));
     PFN_cuTensorMapEncodeTiled_v12000 enc = map_encoder();
@@ -528,7 +528,7 @@ int launch_lean_batch(const PlaneArgs* d_args, const int64_t* d_start, int R, in
         if (blocks == 0) {  // either may be launched
             const int rc = launch_lean_batch_nw<WY, FIELD, HASMP, 8>(d_args, d_start, R, 0, sweep_add, s);
             if (rc) return rc;
-        } else if (lean_warps(blocks) == 8) {
+        } else if (lean_warps(blocks, HASMP ? 0 : LeanCfg<WY, FIELD, HASMP>::MINB) == 8) {
             return launch_lean_batch_nw<WY, FIELD, HASMP, 8>(d_args, d_start, R, blocks, sweep_add, s);
         }
     }

@@ -22,7 +22,16 @@ constexpr int kSMs = 152;
 // and four warps issue fewer.  us per MCS, point field, four warps -> eight: 44 x 76 x 32
 // (96 windows) 27.0 -> 18.6, 76 x 64 x 40 22.8 -> 15.8, 112^3 (448) 29.4 -> 23.4, but
 // 128 x 128 x 64 (480) 30.0 -> 32.5; ensembles of two 48^3, grain field 22.4 -> 15.2.
-inline int lean_warps(int64_t windows) { return windows <= 3 * kSMs ? 8 : 4; }
+// So is a second wave of four-warp windows that comes to no more than a third of the
+// first (`wave`: how many an SM holds; 0 with material points, where it does not pay):
+// ensembles of 200-site grains, 64^3, 128^3 and 64^3 (1344 windows) 67.0 -> 55.9, 2 x 96^3
+// and 2 x 64^3 (1152) 55.3 -> 49.8, 160^3 (1440) 59.5 -> 58.0, but 8 x 64^3 (1536) 59.3 ->
+// 64.1.
+inline int lean_warps(int64_t windows, int wave = 0) {
+    if (windows <= 3 * kSMs) return 8;
+    const int64_t first = (int64_t)wave * kSMs;
+    return windows > first && 100 * windows <= 136 * first ? 8 : 4;
+}
 
 // ---- 2D tiles (tile.cu): cores of 120 x 28 (variant 3) and 120 x 60 (variant 4) ------
 inline int64_t tiles_2d(int64_t Lx, int64_t Ly, int core) { return ((Lx + 119) / 120) * ((Ly + core - 1) / core); }

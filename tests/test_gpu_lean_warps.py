@@ -45,7 +45,8 @@ def test_both_warp_counts_bit_exact(oracle, L, mode):
 
 
 @pytest.mark.parametrize("mode,mp", [("none", False), ("grain", False), ("none", True), ("grain", True), ("point", True)])
-@pytest.mark.parametrize("shapes", [[(34, 30, 6), (64, 28, 4), (2, 2, 2)], [(126, 90, 60), (58, 30, 40), (112, 56, 34)]])
+@pytest.mark.parametrize("shapes", [[(34, 30, 6), (64, 28, 4), (2, 2, 2)], [(126, 90, 60), (58, 30, 40), (112, 56, 34)],
+                                    [(112, 140, 144), (112, 140, 134)]])
 def test_ensembles_bit_exact(oracle, shapes, mode, mp):
     torch, hm = need_gpu()
     kT, members = 0.9, []

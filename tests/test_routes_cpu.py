@@ -34,6 +34,14 @@ def test_few_windows_take_eight_warps(ask):
     assert got == [8] * len(small) + [4] * len(large)
 
 
+def test_a_scant_second_wave_takes_eight_warps(ask):
+    """Ensembles without material points whose four-warp windows (seven an SM) just overflow
+    one wave: 64^3, 128^3 and 64^3 were slower so than they had been with eight warps."""
+    got = ask(*(f"lean_warps({w}, 7)" for w in (456, 576, 960, 1064, 1065, 1152, 1344, 1440, 1536, 1920, 6400)))
+    assert got == [8, 4, 4, 4, 8, 8, 8, 8, 4, 4, 4]
+    assert ask("lean_warps(1344)", "lean_warps(1344, 0)") == [4, 4]
+
+
 def test_tall_tiles_where_short_ones_need_a_second_wave(ask):
     """Lattices of 2.3 to 4.2 million sites that the short tiles swept slower."""
     tall = [(8, 1362, 2300), (8, 1190, 3500), (8, 3002, 1000), (8, 1702, 1702), (8, 2046, 1500), (8, 1502, 2000),
