@@ -83,16 +83,23 @@ __global__ void k_grain_field(FieldArgs a) {
 // consecutive sites at a time, 16 bytes a lane where the array lies on a 16-byte
 // boundary (a thread that scans 32 sites by itself makes every load of a warp touch
 // 32 lines), finds the run starts with four ballots, and a start's run ends at the
-// next one.
-constexpr int kSeg = 2048;  // sites per warp
+// next one.  A warp goes through `seg` sites: 2048 where the chip is full of warps
+// anyhow, down to 128 where they are few and each step is a wait for memory (hp_measure,
+// 500^2: 77 us with 2048, 65 now, 74 with 32 sites a thread; 64^2 54, 44 and 58).
+constexpr int kSeg = 2048;
+int counts_seg(int64_t N) {
+    int seg = 128;
+    while (seg < kSeg && N > (int64_t)seg * 64 * 152) seg *= 2;  // 64 warps an SM
+    return seg;
+}
 
-__global__ void __launch_bounds__(kT) k_counts(const int32_t* __restrict__ q, int64_t N, int32_t G,
+__global__ void __launch_bounds__(kT) k_counts(const int32_t* __restrict__ q, int64_t N, int32_t G, int seg,
                                                unsigned long long* counts, int32_t* bad) {
     const int lane = threadIdx.x & 31;
     const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const bool vec = ((uintptr_t)q & 15u) == 0;
-    const int64_t end = min((w + 1) * kSeg, N);
-    for (int64_t b = w * kSeg; b < end; b += 128) {
+    const int64_t end = min((w + 1) * seg, N);
+    for (int64_t b = w * seg; b < end; b += 128) {
         const int64_t at = b + 4 * lane;
         const int n = (int)min((int64_t)128, end - b);  // sites of this step
         int32_t v[4];
@@ -309,7 +316,10 @@ extern "C" int hp_grain_field(int32_t G, const float* quat, double C11, double C
     return HP_OK;
 }
 
-static unsigned counts_grid(int64_t N) { return (unsigned)(((N + kSeg - 1) / kSeg * 32 + kT - 1) / kT); }
+static unsigned counts_grid(int64_t N) {
+    const int seg = counts_seg(N);
+    return (unsigned)(((N + seg - 1) / seg * 32 + kT - 1) / kT);
+}
 
 extern "C" int hp_grain_counts(hp_handle* h, int64_t* counts, int32_t* alive, void* stream) {
     hp::Range r_("hp_grain_counts");
@@ -322,7 +332,7 @@ extern "C" int hp_grain_counts(hp_handle* h, int64_t* counts, int32_t* alive, vo
     HP_CUDA(cudaMallocAsync((void**)&bad, sizeof(int32_t), s));
     cudaMemsetAsync(bad, 0, sizeof(int32_t), s);
     ::hp::count_launch();
-    k_counts<<<counts_grid(h->lat.N), kT, 0, s>>>(h->q, h->lat.N, G, reinterpret_cast<unsigned long long*>(counts), bad);
+    k_counts<<<counts_grid(h->lat.N), kT, 0, s>>>(h->q, h->lat.N, G, counts_seg(h->lat.N), reinterpret_cast<unsigned long long*>(counts), bad);
     if (alive) {
         cudaMemsetAsync(alive, 0, sizeof(int32_t), s);
         ::hp::count_launch();
@@ -380,7 +390,7 @@ extern "C" int hp_measure(hp_handle* h, int32_t orient_kind, const float* orient
     int32_t* bad = reinterpret_cast<int32_t*>(sm + kSlotBad);
     const int64_t N = h->lat.N;
     ::hp::count_launch();
-    k_counts<<<counts_grid(N), kT, 0, s>>>(h->q, N, G, h->m_counts, bad);
+    k_counts<<<counts_grid(N), kT, 0, s>>>(h->q, N, G, counts_seg(N), h->m_counts, bad);
     ::hp::count_launch();
     k_grain_stats<<<(G + kT - 1) / kT, kT, 0, s>>>(h->m_counts, G, orient_kind, orient,
                                                    h->desc.field_mode == HP_FIELD_GRAIN ? h->table : nullptr,
