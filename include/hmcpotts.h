@@ -425,7 +425,8 @@ typedef struct {
  * testing: x[i] (device double[n]) = the slip of a system with resolved shear
  * at[i] > g[i] (device float[n] each) and k[i] = P:C:P (device double[n]), the
  * root of at - k x = g(gamma + x) for the Voce law of prm (tau0, taus, h0),
- * x = (at - g)/k without hardening.                                          */
+ * x = (at - g)/k without hardening (a sum of two FP32 numbers, relative error near
+ * 2^-46, or FP64 near a tie of the first; with hardening within 1e-10 of the root). */
 HP_API int hp_debug_return_map(const hp_cp_params* prm, const float* at, const float* g, const double* k, int64_t n,
                                double* x, void* stream);
 
@@ -435,7 +436,7 @@ HP_API int hp_cp_reset(const hp_cp_params* prm, hp_cp_state* st, void* stream);
 /* Apply load increments t = t0+1 .. t0+n_incr to every point (Eq. (3), Taylor:
  * total strain t e diag(1,-1/2,-1/2) in the sample frame).  Point p has the
  * orientation quat[4*grain[p]].  Per increment: trial stress, candidate set
- * |tau_alpha| > g, single-slip return map per candidate (FP64 Newton), energies
+ * |tau_alpha| > g, single-slip return map (its FP32 result as FP64 rounds it), energies
  * E_alpha, Boltzmann probabilities (Eq. (1)) and the pick of Eq. (2) with
  * R = u0/2^32 of Philox(seed; p, t, tag 1).  Afterwards, optionally writes
  * sigma (device float[6][P], NULL to skip), w and E_rho (device float[P] each,

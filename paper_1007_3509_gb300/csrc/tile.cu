@@ -535,8 +535,10 @@ int launch_aniso(const PlaneArgs& a, const Aniso& an, cudaStream_t s) {
 
 }  // namespace
 
-// 1024^2, 8 neighbours, Read-Shockley tables: 18.7 us per MCS; 72 us on the per-colour
-// kernel, four launches whose bins took a 64-bit remainder and division each.
+// 1024^2, 8 neighbours, Read-Shockley tables: 18.7 us per MCS; on the per-colour kernel 72
+// us while its bins took a 64-bit remainder and division each, 34 us with the bins above
+// and chained launches (400^2, 50 and 500 sites a grain: 25.8 and 15.1 here, 21.6 and 19.1
+// per colour; 1022^2 36.2 and 23.5, 37.5 and 34.3).
 int tile_launch_aniso(const PlaneArgs& a, const Aniso& an, int field, bool hasmp, int nbr, cudaStream_t s) {
     if (field == HP_FIELD_POINT && hasmp) return nbr == 8 ? launch_aniso<8, 2, true>(a, an, s) : launch_aniso<4, 2, true>(a, an, s);
     if (field == HP_FIELD_GRAIN && !hasmp) return nbr == 8 ? launch_aniso<8, 1, false>(a, an, s) : launch_aniso<4, 1, false>(a, an, s);
