@@ -392,7 +392,8 @@ HP_API int hp_ensemble_autotune(hp_ensemble* e, int32_t n_mcs, float* ms_out, in
  * replicas share each launch (one CTA per replica tile); the n_mcs launches are
  * captured once into a CUDA graph (re-captured when n_mcs or the variant
  * changes) and replayed as one graph launch on `stream`.  Small 2D replicas whose
- * tile variant was not chosen run resident instead, one cluster each.         */
+ * tile variant was not chosen run resident instead, one cluster each, where an
+ * estimate from their shapes favours it.                                      */
 HP_API int hp_ensemble_sweep(hp_ensemble* e, int32_t n_mcs, void* stream);
 
 /* ------------------------------------------------------------------------ */
