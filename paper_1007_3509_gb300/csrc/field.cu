@@ -16,6 +16,7 @@
 #include <string.h>
 
 #include "common.cuh"
+#include "routes.h"
 
 namespace hp {
 namespace {
@@ -83,16 +84,7 @@ __global__ void k_grain_field(FieldArgs a) {
 // consecutive sites at a time, 16 bytes a lane where the array lies on a 16-byte
 // boundary (a thread that scans 32 sites by itself makes every load of a warp touch
 // 32 lines), finds the run starts with four ballots, and a start's run ends at the
-// next one.  A warp goes through `seg` sites: 2048 where the chip is full of warps
-// anyhow, down to 128 where they are few and each step is a wait for memory (hp_measure,
-// 500^2: 77 us with 2048, 65 now, 74 with 32 sites a thread; 64^2 54, 44 and 58).
-constexpr int kSeg = 2048;
-int counts_seg(int64_t N) {
-    int seg = 128;
-    while (seg < kSeg && N > (int64_t)seg * 64 * 152) seg *= 2;  // 64 warps an SM
-    return seg;
-}
-
+// next one.  A warp goes through `seg` sites (counts_seg).
 __global__ void __launch_bounds__(kT) k_counts(const int32_t* __restrict__ q, int64_t N, int32_t G, int seg,
                                                unsigned long long* counts, int32_t* bad) {
     const int lane = threadIdx.x & 31;

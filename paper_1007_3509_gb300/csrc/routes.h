@@ -1,5 +1,5 @@
-// Rules that choose among the sweep kernels by size and shape, and the geometry that
-// they need.  Plain C++ as well as device code, so that they can be checked on the host.
+// Rules that choose among kernels and their splits by size and shape, and the geometry
+// that they need.  Plain C++ as well as device code, so that they can be checked on the host.
 #pragma once
 
 #include <stdint.h>
@@ -127,5 +127,16 @@ struct TileCost {
         return t > floor ? t : floor;
     }
 };
+
+// ---- Grain counts (field.cu) ---------------------------------------------------------------
+// Sites that a warp goes through, 128 at a step: 2048 where the chip is full of warps
+// anyhow (64 an SM), down to 128 where they are few and each step is a wait for memory.
+// hp_measure, us, 2048 sites throughout / now / 32 sites a thread: 500^2 77 / 65 / 74,
+// 250^2 62 / 52 / 61, 64^2 54 / 44 / 58.
+inline int counts_seg(int64_t N) {
+    int seg = 128;
+    while (seg < 2048 && N > (int64_t)seg * 64 * kSMs) seg *= 2;
+    return seg;
+}
 
 }  // namespace hp

@@ -1,5 +1,5 @@
-"""CPU check of the rules that choose among the sweep kernels (csrc/routes.h), compiled by
-themselves for the host."""
+"""CPU check of the rules that choose among kernels and their splits (csrc/routes.h),
+compiled by themselves for the host."""
 import os
 import subprocess
 
@@ -92,3 +92,9 @@ def test_narrow_lattices_go_per_colour(ask):
     tiles = [rule(4, 128, 2000, 1), rule(4, 360, 360, 1), rule(4, 1024, 1024), rule(8, 100, 4000, 1), rule(8, 128, 600),
              rule(8, 128, 128, 0, 1), rule(8, 256, 256, 1)]
     assert ask(*colour, *tiles) == [1] * len(colour) + [0] * len(tiles)
+
+
+def test_small_lattices_are_counted_by_many_warps(ask):
+    """A share of 2048 sites left a 500^2 lattice to 123 warps, one after the other's step."""
+    sizes = [64 ** 2, 250 ** 2, 500 ** 2, 1116 ** 2, 1116 * 1118, 2000 ** 2, 4096 ** 2, 1024 ** 3]
+    assert ask(*(f"counts_seg({n}LL)" for n in sizes)) == [128, 128, 128, 256, 256, 512, 2048, 2048]
